@@ -172,6 +172,7 @@ int crom_destroy(crom_ctx* ctx) {
     free_weights(ctx);
     cudaFree(ctx->partials);
     cudaFree(ctx->counters);
+    cudaFree(ctx->group_counters);
     cudaFree(ctx->targets);
     cudaFree(ctx->qbase);
     cudaFree(ctx->tangent);
@@ -234,13 +235,25 @@ int crom_set_weights(crom_ctx* ctx, const float* params, size_t n, int params_on
     if (count == 0) return cudaSuccess;
     return cudaMemcpy(*dst, src, count * sizeof(float), cudaMemcpyHostToDevice);
   };
-  if ((e = up(&dw.w1, W1, w * in)) != cudaSuccess || (e = up(&dw.b1, B1, w)) != cudaSuccess ||
+  // W_1 [w][in], its transpose [in][w], and the transposed latent columns in FP64 [r][w]
+  std::vector<float> w1(2 * w * in + 2 * (size_t)r * w);
+  memcpy(w1.data(), W1, w * in * sizeof(float));
+  for (int u = 0; u < w; ++u)
+    for (size_t k = 0; k < in; ++k) {
+      const float v = W1[u * in + k];
+      w1[w * in + k * w + u] = v;
+      const double v64 = v;
+      if (k >= (size_t)m) memcpy(&w1[2 * w * in + 2 * ((k - m) * w + u)], &v64, sizeof(double));
+    }
+  if ((e = up(&dw.w1, w1.data(), w1.size())) != cudaSuccess || (e = up(&dw.b1, B1, w)) != cudaSuccess ||
       (e = up(&dw.wt, wt.data(), wt.size())) != cudaSuccess ||
       (e = up(&dw.bh, bh.data(), bh.size())) != cudaSuccess ||
       (e = up(&dw.wout, Wout, w)) != cudaSuccess) {
     free_weights(ctx);
     return cuda_fail(e, "crom_set_weights (upload)");
   }
+  dw.w1t = dw.w1 + w * in;
+  dw.w1q = reinterpret_cast<double*>(dw.w1t + w * in);
   dw.bout = bout;
 
   // f16 images of the tensor-core kernels; left out (those precisions then return

@@ -41,7 +41,9 @@ constexpr int kTcBiasBytes = kTcWidth * 64 * 2;
 
 struct DeviceWeights {
   // FP32 copies for the CUDA-core path.
-  float* w1 = nullptr;    // [width][m+r] row-major
+  float* w1 = nullptr;    // [width][m+r] row-major; w1t and w1q lie in the same allocation
+  float* w1t = nullptr;   // [m+r][width]: transposed
+  double* w1q = nullptr;  // [r][width]: the latent columns, transposed, in FP64
   float* b1 = nullptr;    // [width]
   float* wt = nullptr;    // (hidden-1) x [width(in)][width(out)]: transposed hidden matrices
   float* bh = nullptr;    // (hidden-1) x [width]
@@ -71,6 +73,8 @@ struct crom_ctx {
   size_t partials_cap = 0;     // in doubles
   int* counters = nullptr;     // [n_inst], zero between launches
   size_t counters_cap = 0;
+  int* group_counters = nullptr;  // [n_inst][groups]: completed partial rows per group of chains, zero between launches
+  size_t group_counters_cap = 0;
   double* targets = nullptr;   // [n_samples]: Delta f_j (FP64) from GN iteration 0
   size_t targets_cap = 0;
   double* qbase = nullptr;     // [n_inst][r]: q_n kept for the difference channel

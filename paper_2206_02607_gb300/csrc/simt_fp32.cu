@@ -2,8 +2,12 @@
 // (paper Algorithm 2, App. E.1.1, extended to second order), used by
 // crom_decode, FP32 crom_reconstruct and the plain FP32 crom_step.
 //
-// One CTA = KS threads per hidden unit (blockDim = KS * width) and a tile of S
-// samples.  All channels of a (unit, sample) pair live in one thread, so the
+// Three kernels form the same sums in the same order (bit-identical results):
+// fwd_tile_kernel and fwd_small_kernel (simt_tile.cuh) for many and for few samples, and
+// fwd_fp32_kernel for the shapes neither holds (many channels at the largest widths).
+//
+// fwd_fp32_kernel: one CTA = KS threads per hidden unit (blockDim = KS * width) and a
+// tile of S samples.  All channels of a (unit, sample) pair live in one thread, so the
 // ELU chain rule needs no communication:
 //   z = W h + b;  dz = W dh;  d2z = W d2h
 //   h = s(z);     dh = s'(z) dz;  d2h = s''(z) dz^2 + s'(z) d2z
@@ -11,26 +15,30 @@
 // the transposed hidden matrices are read through L1 (coalesced in the unit index).
 // Each contraction over the width is split in KS slices (one per thread of a unit)
 // whose partial sums are added through shared memory, which shortens the serial
-// dependency chain of the small single-instance problems this path serves.
+// dependency chain.
 //
 // The FP32 step spreads one instance over ceil(|M_i| / S) CTAs.  Each CTA forms
 // its partial normal equations sum_j J_j J_j^T and sum_j J_j rho_j in FP64 from
 // the FP32 Jacobian rows (exact products), writes them to scratch and takes a
-// ticket; the CTA holding the last ticket adds the partials in tile order
-// (deterministic), solves by FP64 Cholesky and updates q (paper §4.3, App. C).
+// ticket; the CTA holding the last ticket adds the partials in a fixed order
+// (finish_cta), solves by FP64 Cholesky and updates q (paper §4.3, App. C).
 // Nothing ever waits on another CTA.
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "crom_internal.h"
 #include "linalg.cuh"
+#include "tc_common.cuh"
 
 namespace crom {
 namespace {
 
 constexpr int kMaxM = 3;
 constexpr int kMaxR = 32;
+constexpr int kSumGroups = 8;  // groups of partial-row chains (finish_cta)
 constexpr int kKSplit = 4;  // threads per hidden unit (width <= 256 -> <= 1024 threads)
 
 enum Mode { kModeDecode = 0, kModeRecon = 1, kModeStep = 2 };
@@ -40,6 +48,8 @@ struct FwdParams {
   // decoder
   int m, r, width, hidden;
   const float* w1;
+  const float* w1t;  // W_1 transposed, [m + r][width]
+  const double* w1q;  // its latent rows in FP64, [r][width]
   const float* b1;
   const float* wt;
   const float* bh;
@@ -75,9 +85,12 @@ struct FwdParams {
   int* status;
   int n_samples;  // length of the sample arrays: every instance's range must lie inside
   double* partials;
-  int max_tiles;
+  int max_tiles;  // partial rows per instance
   int n_entries;
-  int* counters;
+  int PS;         // samples per partial row (divides S)
+  int groups;     // groups the chains of partial rows are dealt to (1: the last CTA adds all)
+  int* counters;        // [n_inst], zero between launches
+  int* group_counters;  // [n_inst][groups], zero between launches
   double* targets;  // Delta f_j per sample (FP64), written at GN iteration 0
   double* qbase;    // q_n per instance, written at GN iteration 0
 };
@@ -168,6 +181,230 @@ __device__ int find_instance(const int* off, int n_inst, int point) {
   return lo;
 }
 
+// ---- shared by the forward kernels: the linear output layer and what a CTA does with it
+
+// outv[t] = w_out . (column t of the last activations), one thread per column, one FMA
+// chain in k; the value channel's columns (t < S with the [channel][sample] order, S > 0;
+// else every C-th) get b_out.
+__device__ __forceinline__ void output_layer(const FwdParams& p, const float* wout, const float* H, int LD, int NP,
+                                             float* outv, int S) {
+  const int W = p.width;
+  for (int t = threadIdx.x; t < NP; t += blockDim.x) {
+    float acc = 0.f;
+#pragma unroll 16
+    for (int k = 0; k < W; ++k) acc = fmaf(wout[k], H[k * LD + t], acc);
+    if (S > 0 ? t < S : t % p.C == 0) acc += p.bout;
+    outv[t] = acc;
+  }
+}
+
+// Entry e of the packed normal equations: (a, b), a <= b, of J^T J in row order, or
+// (a, -1) of J^T rho.
+__device__ __forceinline__ void entry_of(int e, int r, int ntri, int& a, int& b) {
+  if (e < ntri) {
+    // row a starts at a r - a (a - 1) / 2
+    const float t = r + 0.5f;
+    a = (int)(t - sqrtf(t * t - 2.f * e));
+    if (a * r - a * (a - 1) / 2 > e) --a;
+    if ((a + 1) * r - (a + 1) * a / 2 <= e) ++a;
+    b = a + e - (a * r - a * (a - 1) / 2);
+  } else {
+    a = e - ntri;
+    b = -1;
+  }
+}
+// x[0] + x[stride] + .. (n terms, in order), the loads issued ahead of the additions.
+__device__ __forceinline__ double chain_sum(const double* x, int n, size_t stride) {
+  double acc = 0.0;
+  for (int k0 = 0; k0 < n; k0 += 20) {
+    double v[20];
+#pragma unroll
+    for (int k = 0; k < 20; ++k)
+      if (k0 + k < n) v[k] = __ldcg(x + (size_t)(k0 + k) * stride);
+#pragma unroll
+    for (int k = 0; k < 20; ++k)
+      if (k0 + k < n) acc += v[k];
+  }
+  return acc;
+}
+
+// Output channels c of sample s at outv[s * ss + c * cs]: written out (decode,
+// reconstruction), or (step) the residuals, this CTA's partial normal equations and, in
+// the instance's last CTA, their sum and the solve.  rho [S], Amat [r][r + 1], jd [S][r]
+// and red2 ([max(4 width, entries)]) are shared memory.
+//
+// The FP64 sums are formed in one fixed order whatever the tiling: a partial row per
+// p.PS samples (in order of the samples; `total` = the instance's); row t belongs to chain t mod `per` (per =
+// 4 width / entries, at least 1); a chain adds its rows in order, and the chains are
+// added in order.  A call's result therefore does not depend on which kernel ran.
+// FP64 is slow here (64 clocks per warp instruction), so with p.groups > 1 the chains
+// are dealt to that many groups, and the CTA that completes a group's last row adds its
+// chains (into their first rows); the CTA that completes the last group adds the chains.
+__device__ __forceinline__ void finish_cta(const FwdParams& p, const float* outv, int ss, int cs, int inst, int first,
+                                           int ns, int ntiles, int total, double* rho, double* Amat, double* jd,
+                                           double* red2) {
+  __shared__ int s_flag;
+  __shared__ unsigned s_groups;
+  const int tid = threadIdx.x, NT = blockDim.x, m = p.m, r = p.r;
+  if (p.mode == kModeRecon) {
+    for (int s = tid; s < ns; s += NT) p.out[(size_t)blockIdx.y * p.n_pts + first + s] = outv[s * ss];
+    return;
+  }
+  const int n2 = (p.second == kSecondPerK) ? m : (p.second == kSecondLap ? 1 : 0);
+  const int ox = 1 + p.diff, o2 = ox + p.nx, oq = o2 + n2;
+  if (p.mode == kModeDecode) {
+    for (int s = tid; s < ns; s += NT) {
+      const float* c = outv + s * ss;
+      const size_t N = (size_t)p.n_pts, pt = (size_t)(first + s);
+      int row = 0;
+      if (p.want & CROM_WANT_VAL) p.out[(row++) * N + pt] = c[0];
+      if (p.want & CROM_WANT_DX)
+        for (int k = 0; k < m; ++k) p.out[(row++) * N + pt] = c[(ox + k) * cs];
+      if (p.want & CROM_WANT_DXX)
+        for (int k = 0; k < m; ++k) p.out[(row++) * N + pt] = c[(o2 + k) * cs];
+      if (p.want & CROM_WANT_LAP) {
+        float lap = 0.f;
+        for (int k = 0; k < n2; ++k) lap += c[(o2 + k) * cs];
+        p.out[(row++) * N + pt] = lap;
+      }
+      if (p.want & CROM_WANT_DQ)  // r rows, or the one directional row of a tangent decode
+        for (int j = 0; j < p.nq; ++j) p.out[(row++) * N + pt] = c[(oq + j) * cs];
+    }
+    return;
+  }
+
+  // ---- step: residual per sample (Step 2 at iteration 0), partial normal equations
+  for (int i = tid; i < ns * r; i += NT) jd[i] = (double)outv[i / r * ss + (oq + i % r) * cs];
+  for (int s = NT - 1 - tid; s < ns; s += NT) {
+    double res;
+    const float* c = outv + s * ss;
+    const size_t j = (size_t)(first + s);
+    if (p.iter == 0) {
+      double df;
+      const double a = (double)p.alpha[p.coef_per_sample ? j : (size_t)inst];
+      if (p.pde == CROM_PDE_HEAT) {
+        df = p.dt * a * (double)c[o2 * cs];
+      } else {
+        double adv = 0.0;
+        for (int k = 0; k < m; ++k) adv += (double)p.vel[j * m + k] * (double)c[(ox + k) * cs];
+        df = p.dt * (-adv + a * (double)c[o2 * cs]);
+      }
+      p.targets[j] = df;
+      res = -df;  // g(y_j, q^(0)) - f_{n+1}(y_j) with f_{n+1} = g(y_j, q_n) + Delta f_j
+    } else {
+      // g(y_j, q^(k)) - f_{n+1}(y_j) = [g(y_j, q^(k)) - g(y_j, q_n)] - Delta f_j,
+      // the bracket being the difference channel.
+      res = (double)c[cs] - p.targets[j];
+    }
+    rho[s] = res;
+  }
+  __syncthreads();
+  const int ne = p.n_entries, ntri = r * (r + 1) / 2;
+  const int row0 = blockIdx.y * (p.S / p.PS), rows = (ns + p.PS - 1) / p.PS;  // this CTA's partial rows
+  double* base = p.partials + (size_t)inst * p.max_tiles * ne;
+  for (int e = tid; e < ne; e += NT) {
+    int a, b;
+    entry_of(e, r, ntri, a, b);  // (a, b) of J^T J, or (a, -1) of J^T rho
+    for (int t = 0; t < rows; ++t) {
+      double acc = 0.0;
+      const int s1 = min(ns, (t + 1) * p.PS);
+      for (int s = t * p.PS; s < s1; ++s) acc += jd[s * r + a] * (b >= 0 ? jd[s * r + b] : rho[s]);
+      base[(size_t)(row0 + t) * ne + e] = acc;
+    }
+  }
+  const int nrows = (total + p.PS - 1) / p.PS;
+  const int per = max(1, 4 * p.width / ne), chains = min(per, nrows);
+  const int groups = min(p.groups, chains);
+  int* counters = p.counters + inst;  // CTAs, or completed groups
+  // the barrier makes every thread's rows visible to thread 0, whose fence and atomic
+  // publish them (release is cumulative)
+  __syncthreads();
+  if (groups > 1) {
+    int* gcount = p.group_counters + (size_t)inst * p.groups;
+    if (tid < 32) {
+      // lane g: this CTA's rows of group g (chains g, g + groups, ..) and the group's rows in all
+      int mine = 0, all = 0;
+      if (tid < groups) {
+        for (int t = row0; t < row0 + rows; ++t) mine += t % per % groups == tid;
+        for (int j = tid; j < chains; j += groups) all += (nrows - j + per - 1) / per;
+      }
+      __threadfence();
+      const bool last = mine > 0 && atomicAdd(&gcount[tid], mine) == all - mine;
+      const unsigned d = __ballot_sync(0xffffffffu, last);
+      __threadfence();
+      if (tid == 0) s_groups = d;
+    }
+    __syncthreads();
+    const unsigned done = s_groups;
+    if (!done) return;
+    for (int g = 0; g < groups; ++g) {
+      if (!(done >> g & 1)) continue;
+      const int nc = (chains - g + groups - 1) / groups;
+      for (int i = tid; i < nc * ne; i += NT) {
+        const int j = g + i / ne * groups;
+        double* row = base + (size_t)j * ne + i % ne;
+        *row = chain_sum(row, (nrows - j + per - 1) / per, (size_t)per * ne);
+      }
+      if (tid == 0) gcount[g] = 0;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      const int n = __popc(done);
+      __threadfence();
+      s_flag = atomicAdd(counters, n) == groups - n;
+      __threadfence();
+    }
+  } else if (tid == 0) {
+    __threadfence();
+    s_flag = atomicAdd(counters, 1) == ntiles - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!s_flag) return;
+
+  // ---- last CTA of the instance: add the chains in order, solve, update q
+  if (groups <= 1) {
+    for (int i = tid; i < chains * ne; i += NT) {
+      const int e = i % ne, j = i / ne;
+      red2[i] = chain_sum(base + (size_t)j * ne + e, (nrows - j + per - 1) / per, (size_t)per * ne);
+    }
+    __syncthreads();
+  }
+  for (int e = tid; e < ne; e += NT) {
+    double acc;
+    if (groups > 1) {
+      acc = chain_sum(base + e, chains, (size_t)ne);
+    } else {
+      acc = 0.0;
+      for (int j = 0; j < chains; ++j) acc += red2[j * ne + e];
+    }
+    int a, b;
+    entry_of(e, r, ntri, a, b);
+    if (b >= 0) {
+      Amat[a * (r + 1) + b] = acc;
+      Amat[b * (r + 1) + a] = acc;
+    } else {
+      Amat[a * (r + 1) + r] = -acc;  // right-hand side -J^T rho
+    }
+  }
+  __syncthreads();
+  if (tid < 32) {
+    // Cholesky A = L L^T and the two triangular solves, spread over one warp
+    __shared__ double s_invd[kMaxR];
+    const int st = chol_solve_warp(Amat, s_invd, r, tid);
+    if (st == CROM_OK && tid < r) {
+      if (p.iter == 0) p.qbase[(size_t)inst * r + tid] = p.qio[(size_t)inst * r + tid];
+      p.qio[(size_t)inst * r + tid] += Amat[tid * (r + 1) + r];
+    }
+    if (tid == 0) {
+      p.status[inst] = st;
+      counters[0] = 0;
+    }
+  }
+}
+
+#include "simt_tile.cuh"
+
 // kJvp: the tangent-velocity decode, whose directional channel is seeded per
 // instance (kept out of the other instantiation, whose register budget it would
 // change).
@@ -192,7 +429,6 @@ __device__ __forceinline__ void fwd_fp32_body(const FwdParams& p) {
   float* outv = xs + S * m;                               // [NPP]
   // [KS][W][16] split-K partial sums (16-byte aligned: also reused as doubles)
   float* red = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(outv + NPP) + 15) & ~uintptr_t(15));
-  __shared__ int s_flag;
 
   // ---- which samples does this CTA own?
   int inst = 0, first = 0, ns = 0, ntiles = 0, msz = 0;
@@ -322,141 +558,12 @@ __device__ __forceinline__ void fwd_fp32_body(const FwdParams& p) {
     float* tmp = Hin; Hin = Hout; Hout = tmp;
   }
 
-  // ---- linear output layer: one thread per (sample, channel) column
-  for (int t = tid; t < NP; t += NT) {
-    float acc = 0.f;
-    for (int k = 0; k < W; ++k) acc = fmaf(__ldg(&p.wout[k]), Hin[k * LD + t], acc);
-    if (t % C == 0) acc += p.bout;
-    outv[t] = acc;
-  }
+  output_layer(p, p.wout, Hin, LD, NP, outv, 0);
   __syncthreads();
-
-  if (p.mode == kModeRecon) {
-    if (tid < ns) p.out[(size_t)blockIdx.y * p.n_pts + first + tid] = outv[tid * C];
-    return;
-  }
-  const int n2 = (p.second == kSecondPerK) ? m : (p.second == kSecondLap ? 1 : 0);
-  const int ox = 1 + p.diff, o2 = ox + p.nx, oq = o2 + n2;
-  if (p.mode == kModeDecode) {
-    for (int s = tid; s < ns; s += NT) {
-      const float* c = outv + s * C;
-      const size_t N = (size_t)p.n_pts, pt = (size_t)(first + s);
-      int row = 0;
-      if (p.want & CROM_WANT_VAL) p.out[(row++) * N + pt] = c[0];
-      if (p.want & CROM_WANT_DX)
-        for (int k = 0; k < m; ++k) p.out[(row++) * N + pt] = c[ox + k];
-      if (p.want & CROM_WANT_DXX)
-        for (int k = 0; k < m; ++k) p.out[(row++) * N + pt] = c[o2 + k];
-      if (p.want & CROM_WANT_LAP) {
-        float lap = 0.f;
-        for (int k = 0; k < n2; ++k) lap += c[o2 + k];
-        p.out[(row++) * N + pt] = lap;
-      }
-      if (p.want & CROM_WANT_DQ)  // r rows, or the one directional row of a tangent decode
-        for (int j = 0; j < p.nq; ++j) p.out[(row++) * N + pt] = c[oq + j];
-    }
-    return;
-  }
-
-  // ---- step: residual per sample (Step 2 at iteration 0), partial normal equations
-  const int t = blockIdx.y;
-  for (int s = tid; s < S; s += NT) {
-    double res = 0.0;
-    if (s < ns) {
-      const float* c = outv + s * C;
-      const size_t j = (size_t)(first + s);
-      if (p.iter == 0) {
-        double df;
-        const double a = (double)p.alpha[p.coef_per_sample ? j : (size_t)inst];
-        if (p.pde == CROM_PDE_HEAT) {
-          df = p.dt * a * (double)c[o2];
-        } else {
-          double adv = 0.0;
-          for (int k = 0; k < m; ++k) adv += (double)p.vel[j * m + k] * (double)c[ox + k];
-          df = p.dt * (-adv + a * (double)c[o2]);
-        }
-        p.targets[j] = df;
-        res = -df;  // g(y_j, q^(0)) - f_{n+1}(y_j) with f_{n+1} = g(y_j, q_n) + Delta f_j
-      } else {
-        // g(y_j, q^(k)) - f_{n+1}(y_j) = [g(y_j, q^(k)) - g(y_j, q_n)] - Delta f_j,
-        // the bracket being the difference channel.
-        res = (double)c[1] - p.targets[j];
-      }
-    }
-    rho[s] = res;
-  }
-  __syncthreads();
-  double* part = p.partials + ((size_t)inst * p.max_tiles + t) * p.n_entries;
-  for (int e = tid; e < p.n_entries; e += NT) {
-    const int ntri = r * (r + 1) / 2;
-    double acc = 0.0;
-    if (e < ntri) {
-      int a = 0, rem = e;
-      while (rem >= r - a) { rem -= r - a; ++a; }
-      const int b = a + rem;
-      for (int s = 0; s < ns; ++s)
-        acc += (double)outv[s * C + oq + a] * (double)outv[s * C + oq + b];
-    } else {
-      const int a = e - ntri;
-      for (int s = 0; s < ns; ++s) acc += (double)outv[s * C + oq + a] * rho[s];
-    }
-    part[e] = acc;
-  }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    const int ticket = atomicAdd(&p.counters[inst], 1);
-    s_flag = (ticket == ntiles - 1);
-  }
-  __syncthreads();
-  if (!s_flag) return;
-  __threadfence();
-
-  // ---- last CTA of the instance: reduce partials in a fixed order, solve, update q
-  // (thread (j, e) adds the tiles j, j + per, ... of entry e; then the per partial
-  // sums of each entry are added in order).
-  const double* base = p.partials + (size_t)inst * p.max_tiles * p.n_entries;
-  const int ne = p.n_entries;
-  const int per = NT >= ne ? NT / ne : 1;
-  double* red2 = reinterpret_cast<double*>(red);  // [per][ne]
-  for (int idx = tid; idx < per * ne; idx += NT) {
-    const int e = idx % ne, j = idx / ne;
-    double acc = 0.0;
-    for (int tt = j; tt < ntiles; tt += per) acc += __ldcg(&base[(size_t)tt * ne + e]);
-    red2[(size_t)j * ne + e] = acc;
-  }
-  __syncthreads();
-  for (int e = tid; e < ne; e += NT) {
-    double acc = 0.0;
-    for (int j = 0; j < per; ++j) acc += red2[(size_t)j * ne + e];
-    const int ntri = r * (r + 1) / 2;
-    if (e < ntri) {
-      int a = 0, rem = e;
-      while (rem >= r - a) { rem -= r - a; ++a; }
-      const int b = a + rem;
-      Amat[a * (r + 1) + b] = acc;
-      Amat[b * (r + 1) + a] = acc;
-    } else {
-      Amat[(e - ntri) * (r + 1) + r] = -acc;  // right-hand side -J^T rho
-    }
-  }
-  __syncthreads();
-  if (tid < 32) {
-    // Cholesky A = L L^T and the two triangular solves, spread over one warp
-    __shared__ double s_invd[kMaxR];
-    const int st = chol_solve_warp(Amat, s_invd, r, tid);
-    if (st == CROM_OK && tid < r) {
-      if (p.iter == 0) p.qbase[(size_t)inst * r + tid] = p.qio[(size_t)inst * r + tid];
-      p.qio[(size_t)inst * r + tid] += Amat[tid * (r + 1) + r];
-    }
-    if (tid == 0) {
-      p.status[inst] = st;
-      p.counters[inst] = 0;
-    }
-  }
+  finish_cta(p, outv, C, 1, inst, first, ns, ntiles, msz, rho, Amat, qs, reinterpret_cast<double*>(red));
 }
 
-__global__ void fwd_fp32_kernel(FwdParams p) { fwd_fp32_body<false>(p); }
+__global__ void __launch_bounds__(1024) fwd_fp32_kernel(FwdParams p) { fwd_fp32_body<false>(p); }
 // up to 1024 threads per CTA: the bound keeps it within 64 registers
 __global__ void __launch_bounds__(1024) fwd_fp32_jvp_kernel(FwdParams p) { fwd_fp32_body<true>(p); }
 
@@ -473,15 +580,97 @@ size_t fwd_smem_bytes(int W, int S, int C, int m, int r, int* LD_out) {
   return b + 64;
 }
 
-cudaError_t launch_fwd(FwdParams& p, dim3 grid, cudaStream_t s) {
-  size_t smem = fwd_smem_bytes(p.width, p.S, p.C, p.m, p.r, &p.LD);
-  auto kernel = p.jvp_seed ? fwd_fp32_jvp_kernel : fwd_fp32_kernel;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+// Which of the forward kernels runs a launch.
+enum FwdKernel { kFwdGeneral = 0, kFwdTile2, kFwdTile3, kFwdSmall };
+constexpr size_t kMaxSmem = 227 * 1024;
+
+cudaError_t launch_fwd(FwdParams& p, FwdKernel kind, dim3 grid, cudaStream_t s) {
+  const int W = p.width;
+  auto go = [&](auto kernel, int threads, size_t smem) -> cudaError_t {
+    if (smem > 48 * 1024) {
+      cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+    }
+    kernel<<<grid, threads, smem, s>>>(p);
+    return cudaGetLastError();
+  };
+  const bool siren = p.act == CROM_ACT_SIREN;
+  if (kind == kFwdTile2 || kind == kFwdTile3) {
+    p.LD = tile_ld(p.C, p.S);
+    const size_t smem = tile_smem_bytes(W, p.S, p.C, p.m, p.r);
+    const int tq = kind == kFwdTile2 ? 2 : 3, threads = tile_threads(W, p.S, p.C, tq);
+    auto tile = [&](auto k68, auto k132) { return p.LD == 68 ? go(k68, threads, smem) : go(k132, threads, smem); };
+    if (tq == 2)
+      return siren ? tile(fwd_tile_kernel<2, true, 68>, fwd_tile_kernel<2, true, 132>)
+                   : tile(fwd_tile_kernel<2, false, 68>, fwd_tile_kernel<2, false, 132>);
+    return siren ? tile(fwd_tile_kernel<3, true, 68>, fwd_tile_kernel<3, true, 132>)
+                 : tile(fwd_tile_kernel<3, false, 68>, fwd_tile_kernel<3, false, 132>);
   }
-  kernel<<<grid, p.width * kKSplit, smem, s>>>(p);
-  return cudaGetLastError();
+  if (kind != kFwdGeneral) {
+    // more threads than the products need fetch the weights and share the activation passes
+    const size_t smem = small_smem_bytes(W, p.S, p.C, p.m, p.r, p.hidden);
+    auto small = [&](auto k64, auto k128, auto any) {
+      return W == 64 ? go(k64, kSmallThreads, smem) : W == 128 ? go(k128, kSmallThreads, smem) : go(any, kSmallThreads, smem);
+    };
+    return small(fwd_small_kernel<64>, fwd_small_kernel<128>, fwd_small_kernel<0>);
+  }
+  const size_t smem = fwd_smem_bytes(W, p.S, p.C, p.m, p.r, &p.LD);
+  return p.jvp_seed ? go(fwd_fp32_jvp_kernel, W * kKSplit, smem) : go(fwd_fp32_kernel, W * kKSplit, smem);
+}
+
+// The tile kernel's variant for S samples of C channels, or kFwdGeneral if none fits.
+FwdKernel tile_variant(int W, int S, int C, int m, int r) {
+  if (tile_ld(C, S) == 0 || tile_smem_bytes(W, S, C, m, r) > kMaxSmem) return kFwdGeneral;
+  // three quads per thread where they give whole 128-thread CTAs of 8 samples
+  if (S == 8 && tile_threads(W, S, C, 3) <= 128) return kFwdTile3;
+  if (tile_threads(W, S, C, 2) <= 256) return kFwdTile2;
+  if (tile_threads(W, S, C, 3) <= 256) return kFwdTile3;
+  return kFwdGeneral;
+}
+// Samples per CTA of the tile kernel for `sets` groups of n samples: 8 with three quads
+// per thread if that fills 128 threads, else the largest multiple of 4 with at most 128
+// threads (256 for a lone value channel), in any case two CTAs per SM.
+FwdKernel tile_plan(const crom_ctx* ctx, long long sets, long long n, int C, int* S) {
+  const int W = ctx->desc.width, m = ctx->desc.m, r = ctx->desc.r;
+  auto many = [&](int t) { return t == 4 || sets * ((n + t - 1) / t) >= 2LL * ctx->num_sms; };
+  const int t3 = tile_threads(W, 8, C, 3);
+  if (t3 > 96 && t3 <= 128 && many(8) && tile_variant(W, 8, C, m, r) != kFwdGeneral) {
+    *S = 8;
+    return kFwdTile3;
+  }
+  for (int t = 64; t >= 4; t -= 4) {
+    if (t > 4 && (tile_threads(W, t, C, 2) > (C == 1 ? 256 : 128) || !many(t))) continue;
+    const FwdKernel k = tile_variant(W, t, C, m, r);
+    if (k != kFwdGeneral) {
+      *S = t;
+      return k;
+    }
+  }
+  return kFwdGeneral;
+}
+// Whether the latency kernel holds S samples of C channels.
+bool small_fits(int W, int S, int C, int m, int r, int hidden) {
+  return S * C <= kSmallLD - 4 && small_smem_bytes(W, S, C, m, r, hidden) <= kMaxSmem &&
+         small_gemm_threads(W, S, C) <= kSmallThreads;
+}
+
+int pick_samples(int W, int C, int m, int r, int want);
+
+// Kernel and samples per CTA for `sets` groups of n points with C channels (decode and
+// reconstruction): the tile kernel once its smallest tiles (4 samples) give every SM
+// one, below that the latency kernel, two samples per CTA where one would not fit the
+// GPU at once (200 samples of a 2D step: 72 us with two, 96 us with one per CTA).
+FwdKernel plan_points(const crom_ctx* ctx, long long sets, long long n, int C, int general_want, int* S) {
+  const int W = ctx->desc.width, m = ctx->desc.m, r = ctx->desc.r;
+  if (sets * ((n + 3) / 4) >= ctx->num_sms) {
+    const FwdKernel k = tile_plan(ctx, sets, n, C, S);
+    if (k != kFwdGeneral) return k;
+  } else {
+    for (*S = sets * n > ctx->num_sms ? 2 : 1; *S >= 1; --*S)
+      if (small_fits(W, *S, C, m, r, ctx->desc.hidden)) return kFwdSmall;
+  }
+  *S = pick_samples(W, C, m, r, general_want);
+  return kFwdGeneral;
 }
 
 void fill_decoder(FwdParams& p, const crom_ctx* ctx) {
@@ -490,6 +679,8 @@ void fill_decoder(FwdParams& p, const crom_ctx* ctx) {
   p.width = ctx->desc.width;
   p.hidden = ctx->desc.hidden;
   p.w1 = ctx->w.w1;
+  p.w1t = ctx->w.w1t;
+  p.w1q = ctx->w.w1q;
   p.b1 = ctx->w.b1;
   p.wt = ctx->w.wt;
   p.bh = ctx->w.bh;
@@ -540,7 +731,7 @@ cudaError_t launch_tangent_fp32(const crom_ctx* ctx, int n_inst, const double* q
   p.second = kSecondNone;
   p.nq = 1;
   p.C = ChannelSet{p.nx, p.second, p.nq}.count(p.m);
-  p.S = pick_samples(p.width, p.C, p.m, p.r, 8);
+  const FwdKernel kind = plan_points(ctx, 1, n_pts, p.C, 8, &p.S);
   p.q = q;
   p.off = pt_off;
   p.x = x;
@@ -550,7 +741,7 @@ cudaError_t launch_tangent_fp32(const crom_ctx* ctx, int n_inst, const double* q
   p.want = CROM_WANT_DQ;
   p.jvp_seed = seed;
   dim3 grid((n_pts + p.S - 1) / p.S, 1);
-  return launch_fwd(p, grid, s);
+  return launch_fwd(p, kind, grid, s);
 }
 
 cudaError_t launch_decode_fp32(const crom_ctx* ctx, int n_inst, const double* q, const int* pt_off,
@@ -563,7 +754,7 @@ cudaError_t launch_decode_fp32(const crom_ctx* ctx, int n_inst, const double* q,
   p.second = (want & CROM_WANT_DXX) ? kSecondPerK : ((want & CROM_WANT_LAP) ? kSecondLap : kSecondNone);
   p.nq = (want & CROM_WANT_DQ) ? p.r : 0;
   p.C = ChannelSet{p.nx, p.second, p.nq}.count(m);
-  p.S = pick_samples(p.width, p.C, m, p.r, 8);
+  const FwdKernel kind = plan_points(ctx, 1, n_pts, p.C, 8, &p.S);
   p.q = q;
   p.off = pt_off;
   p.x = x;
@@ -572,7 +763,7 @@ cudaError_t launch_decode_fp32(const crom_ctx* ctx, int n_inst, const double* q,
   p.out = out;
   p.want = want;
   dim3 grid((n_pts + p.S - 1) / p.S, 1);
-  return launch_fwd(p, grid, s);
+  return launch_fwd(p, kind, grid, s);
 }
 
 cudaError_t launch_recon_fp32(const crom_ctx* ctx, int n_codes, const double* q, int n_pts,
@@ -584,14 +775,14 @@ cudaError_t launch_recon_fp32(const crom_ctx* ctx, int n_codes, const double* q,
   p.second = kSecondNone;
   p.nq = 0;
   p.C = 1;
-  p.S = 32;
+  const FwdKernel kind = plan_points(ctx, n_codes, n_pts, 1, 32, &p.S);
   p.q = q;
   p.x = x;
   p.n_pts = n_pts;
   p.n_inst = n_codes;
   p.out = out;
   dim3 grid((n_pts + p.S - 1) / p.S, n_codes);
-  return launch_fwd(p, grid, s);
+  return launch_fwd(p, kind, grid, s);
 }
 
 // Samples per CTA of the FP32 step: enough CTAs to cover the GPU at least twice
@@ -602,6 +793,23 @@ int step_samples_per_cta(const crom_ctx* ctx, int n_inst, int max_samples) {
   int S = 4;
   while (S > 1 && (long long)n_inst * ((max_samples + S - 1) / S) < 2LL * ctx->num_sms) S >>= 1;
   return pick_samples(ctx->desc.width, C0, m, r, S);
+}
+
+// Kernel, samples per CTA (S) and per partial row (PS, which bounds the grid and the
+// scratch, and fixes the order of the FP64 sums) of the FP32 step.
+FwdKernel plan_step(const crom_ctx* ctx, int n_inst, int max_samples, int* S, int* PS) {
+  const int W = ctx->desc.width, m = ctx->desc.m, r = ctx->desc.r;
+  const int C0 = ChannelSet{m, kSecondLap, r}.count(m);
+  *PS = step_samples_per_cta(ctx, n_inst, max_samples);
+  if ((long long)n_inst * (((long long)max_samples + 3) / 4) >= ctx->num_sms) {
+    const FwdKernel k = tile_plan(ctx, n_inst, max_samples, C0, S);
+    if (k != kFwdGeneral) return k;
+  } else {
+    for (*S = (long long)n_inst * max_samples > ctx->num_sms ? 2 : 1; *S >= 1; --*S)
+      if (*S % *PS == 0 && small_fits(W, *S, C0, m, r, ctx->desc.hidden)) return kFwdSmall;
+  }
+  *S = *PS;
+  return kFwdGeneral;
 }
 
 int step_fp32_max_tiles(const crom_ctx* ctx, int n_inst, int max_samples) {
@@ -618,8 +826,9 @@ cudaError_t launch_step_fp32(crom_ctx* ctx, const crom_step_desc* step, int n_in
   p.mode = kModeStep;
   fill_decoder(p, ctx);
   const int m = p.m, r = p.r;
-  const int S = step_samples_per_cta(ctx, n_inst, max_samples);
-  const int max_tiles = (max_samples + S - 1) / S;
+  int S, PS;
+  const FwdKernel kind = plan_step(ctx, n_inst, max_samples, &S, &PS);
+  const int max_tiles = (max_samples + PS - 1) / PS;  // partial rows per instance
   const int n_entries = r * (r + 1) / 2 + r;
 
   // Scratch: partial normal equations, per-instance tickets, per-sample targets.
@@ -643,6 +852,21 @@ cudaError_t launch_step_fp32(crom_ctx* ctx, const crom_step_desc* step, int n_in
     e = cudaMemset(ctx->counters, 0, (size_t)n_inst * sizeof(int));
     if (e != cudaSuccess) return e;
     ctx->counters_cap = n_inst;
+  }
+  // the chains of partial rows in groups (finish_cta): for few instances of many rows,
+  // whose last CTA would be alone with the sums
+  const int groups = kind == kFwdSmall && max_tiles > 16 ? kSumGroups : 1;
+  if (groups > 1 && (size_t)n_inst * groups > ctx->group_counters_cap) {
+    if (ctx->group_counters) cudaFree(ctx->group_counters);
+    ++ctx->scratch_gen;
+    ctx->group_counters = nullptr;
+    ctx->group_counters_cap = 0;
+    const size_t n = (size_t)n_inst * groups;
+    cudaError_t e = cudaMalloc(&ctx->group_counters, n * sizeof(int));
+    if (e != cudaSuccess) return e;
+    e = cudaMemset(ctx->group_counters, 0, n * sizeof(int));
+    if (e != cudaSuccess) return e;
+    ctx->group_counters_cap = n;
   }
   if ((size_t)n_samples > ctx->targets_cap) {
     if (ctx->targets) cudaFree(ctx->targets);
@@ -680,10 +904,13 @@ cudaError_t launch_step_fp32(crom_ctx* ctx, const crom_step_desc* step, int n_in
   p.max_tiles = max_tiles;
   p.n_entries = n_entries;
   p.counters = ctx->counters;
+  p.PS = PS;
+  p.groups = groups;
+  p.group_counters = ctx->group_counters;
   p.targets = ctx->targets;
   p.qbase = ctx->qbase;
   if (max_tiles > 65535) return cudaErrorInvalidValue;
-  dim3 grid(n_inst, max_tiles);
+  dim3 grid(n_inst, (max_samples + S - 1) / S);
   for (int it = 0; it < step->gn_iters; ++it) {
     // Iteration 0: value, dg/dx_k, Laplacian, dg/dq at q_n.  Later iterations:
     // value and dg/dq at q^(k) plus the difference channel h(q^(k)) - h(q_n).
@@ -693,7 +920,7 @@ cudaError_t launch_step_fp32(crom_ctx* ctx, const crom_step_desc* step, int n_in
     p.second = (it == 0) ? kSecondLap : kSecondNone;
     p.nq = r;
     p.C = 1 + p.diff + ChannelSet{p.nx, p.second, p.nq}.count(m) - 1;
-    cudaError_t e = launch_fwd(p, grid, s);
+    cudaError_t e = launch_fwd(p, kind, grid, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -758,8 +985,9 @@ cudaError_t launch_step_fp32_noalloc(const crom_ctx* ctx, const crom_step_desc* 
   p.mode = kModeStep;
   fill_decoder(p, ctx);
   const int m = p.m, r = p.r;
-  const int S = step_samples_per_cta(ctx, n_inst, max_samples);
-  const int max_tiles = (max_samples + S - 1) / S;
+  int S, PS;
+  const FwdKernel kind = plan_step(ctx, n_inst, max_samples, &S, &PS);
+  const int max_tiles = (max_samples + PS - 1) / PS;  // partial rows per instance
   const int n_entries = r * (r + 1) / 2 + r;
   // layout inside the static array
   const size_t off_cnt = 0;
@@ -792,9 +1020,11 @@ cudaError_t launch_step_fp32_noalloc(const crom_ctx* ctx, const crom_step_desc* 
   p.max_tiles = max_tiles;
   p.n_entries = n_entries;
   p.counters = reinterpret_cast<int*>(b + off_cnt);
+  p.PS = PS;
+  p.groups = 1;
   p.targets = reinterpret_cast<double*>(b + off_tgt);
   p.qbase = reinterpret_cast<double*>(b + off_qb);
-  dim3 grid(n_inst, max_tiles);
+  dim3 grid(n_inst, (max_samples + S - 1) / S);
   for (int it = 0; it < step->gn_iters; ++it) {
     p.iter = it;
     p.diff = (it == 0) ? 0 : 1;
@@ -802,7 +1032,7 @@ cudaError_t launch_step_fp32_noalloc(const crom_ctx* ctx, const crom_step_desc* 
     p.second = (it == 0) ? kSecondLap : kSecondNone;
     p.nq = r;
     p.C = 1 + p.diff + ChannelSet{p.nx, p.second, p.nq}.count(m) - 1;
-    e = launch_fwd(p, grid, s);
+    e = launch_fwd(p, kind, grid, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
