@@ -216,6 +216,9 @@ cudaError_t launch_step_fp32_noalloc(const crom_ctx* ctx, const crom_step_desc* 
 // Full-order model stencils (fom.cu).
 cudaError_t launch_fom(int kind, int n_batch, int nx, int ny, const float* coef, const float* ax, const float* ay,
                        double dt, int n_steps, float* u, float* tmp, cudaStream_t s);
+// All n_steps in one launch (fom_fused.cu); *done = false where the size is not served.
+cudaError_t launch_fom_fused(int kind, int n_batch, int nx, const float* coef, const float* ax, const float* ay,
+                             double dt, int n_steps, float* u, cudaStream_t s, bool* done);
 
 // Tensor-core launches (tc_step.cu, tc_recon.cu).
 // lo_parts: 1 for F16X2 (activations as f16 hi + lo parts), 0 for F16 (hi parts only)
