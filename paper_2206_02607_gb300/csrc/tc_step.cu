@@ -1,9 +1,10 @@
 // Batched latent step on the tcgen05 tensor cores (crom_step, CROM_PREC_F16X2).
 //
-// One persistent launch per step, one CTA per SM holding the decoder's bf16
+// One persistent launch per step, one CTA per SM holding the decoder's f16
 // hidden matrices in shared memory.  The CTA runs four independent groups of 128
 // threads; each group takes whole instances from a queue ordered by |M_i|
-// (largest first) and has its own 64-column operand block, 128 TMEM columns,
+// (largest first; few or uneven instances instead have their tiles dealt to all groups,
+// one launch per Gauss-Newton iteration: run_iteration and split_wanted) and has its own 64-column operand block, 128 TMEM columns,
 // mbarrier and named barrier, so the UMMAs of one group overlap the CUDA-core
 // epilogues of the others.  Inside a group, hidden unit u is TMEM lane u and
 // thread u of the group.
@@ -122,7 +123,15 @@ struct StepParams {
   // [rows][n_samples]; the output row of each channel, -1 where not wanted
   float* dec_out;
   int row_val, row_dx, row_lap, row_dq;
+  // split mode (kIterFirst, kIterLater): one launch per Gauss-Newton iteration
+  double* qbase;   // [n_inst][r]: q_n, written by iteration 0's solve
+  double* rows;    // [tiles][entries]: every tile's normal-equation terms
+  int rows_cap;    // tiles that rows holds
+  int* counters;   // [n_inst]: tiles done, zero between launches
 };
+// What an instantiation of the kernel does: whole steps (instances from a queue), Step 1
+// alone, or one Gauss-Newton iteration with the instances' tiles dealt to all groups.
+enum Mode { kStep = 0, kDecode = 1, kIterFirst = 2, kIterLater = 3 };
 // Points per work item of the decode mode (a chunk may span several instances).
 constexpr int kDecChunk = 256;
 
@@ -130,6 +139,7 @@ struct __align__(16) Shared {
   uint64_t bar_w;
   uint32_t tmem_base;
   int pad;
+  int part[kThreads / 32];
   float w1x[2][kTcWidth];
   float bh[4][kTcWidth];
   float wout[kTcWidth];
@@ -347,6 +357,7 @@ struct Lane {
 struct Own {
   int ea[2], eb[2];
   double acc[2];
+  double* row;  // split mode: where the tile's terms go instead of into acc
 };
 
 // One UMMA stage of the group: fence the epilogue's shared-memory writes, meet,
@@ -456,7 +467,7 @@ __device__ __forceinline__ void sig1(const Lane& c, const Group* G, float cc, in
 // kSm..2kSm-1), the Jacobian projection and these samples' share of J^T J, J^T rho
 // (and rho^T rho for the line search).  s'(z_l) of hidden layer l + 2 is read from
 // TMEM column kSig + l * kSS + slot.
-template <int kM, int kSm, int kSS, bool kLoP, bool kDec = false>
+template <int kM, int kSm, int kSS, bool kLoP, Mode kMode>
 __device__ __forceinline__ bool reverse_tile(Lane& c, const StepParams& p, int j0, int ns, Own& o) {
   constexpr int kPer = kSm / kTPU;
   constexpr int kC = kPer < 8 ? kPer : 8;
@@ -515,7 +526,7 @@ __device__ __forceinline__ bool reverse_tile(Lane& c, const StepParams& p, int j
     }
   }
   group_sync(c.g);
-  if constexpr (kDec) {  // decode mode: dg/dq rows of the tile's samples (hi + lo parts)
+  if constexpr (kMode == kDecode) {  // decode mode: dg/dq rows of the tile's samples (hi + lo parts)
     const int n = ns * p.r;
     for (int e = c.gt; e < n; e += kGT) {
       const int jq = e / ns, sq = e % ns;
@@ -523,13 +534,19 @@ __device__ __forceinline__ bool reverse_tile(Lane& c, const StepParams& p, int j
       if (kLoP) v = __fadd_rn(v, jrow(G, 1, sq)[jq]);
       p.dec_out[(size_t)(p.row_dq + jq) * p.n_samples + j0 + sq] = v;
     }
-    return true;
   }
   // ---------------- this tile's normal-equation terms
 #pragma unroll
-  for (int e = 0; e < 2; ++e) {
+  for (int e = 0; kMode != kDecode && e < 2; ++e) {
     const int ea = o.ea[e], eb = o.eb[e];
-    if (ea >= 0) {
+    if (kMode >= kIterFirst) {
+      if (ea >= 0) {
+        const float* a0 = jrow(G, 0, 0) + ea;
+        const float* a1 = jrow(G, 1, 0) + ea;
+        o.row[c.gt + e * kGT] = eb >= 0 ? dot_exact<kLoP, kLoP>(a0, a1, 16, jrow(G, 0, 0) + eb, jrow(G, 1, 0) + eb, 16, ns)
+                                        : dot_exact<kLoP, false>(a0, a1, 16, G->rho, G->zero, 1, ns);
+      }
+    } else if (ea >= 0) {
       const float* a0 = jrow(G, 0, 0) + ea;
       const float* a1 = jrow(G, 1, 0) + ea;
       if (eb >= 0) o.acc[e] += dot_exact<kLoP, kLoP>(a0, a1, 16, jrow(G, 0, 0) + eb, jrow(G, 1, 0) + eb, 16, ns);
@@ -547,7 +564,7 @@ __device__ __forceinline__ bool reverse_tile(Lane& c, const StepParams& p, int j
 // (coordinates xs, residual rho, and the TMEM columns kSig + l * kSS + slot that keep
 // s'(z) of hidden layer l + 2 for the reverse pass), so that two tiles of iteration
 // 0 can share one reverse pass.
-template <int kM, int kSm, bool kFirst, int kSS, bool kLoP, bool kDec = false>
+template <int kM, int kSm, bool kFirst, int kSS, bool kLoP, Mode kMode>
 __device__ __forceinline__ bool forward_tile(Lane& c, const StepParams& p, int j0, int so, int ns, float alpha) {
   constexpr int kCh = kFirst ? 2 + kM : 2;  // iteration 0: v, dx_1..dx_m, Lap; later: v(q^(k)), diff
   constexpr int kN = kCh * kSm;             // hi columns 0..kN-1, lo columns kLo..kLo+kN-1
@@ -645,7 +662,7 @@ __device__ __forceinline__ bool forward_tile(Lane& c, const StepParams& p, int j
         for (int ch = 0; ch < kCh; ++ch) {
           // step, iteration 0: the gradient channels only for advection, the Laplacian
           // always; later: the difference channel; decode: the requested channels
-          const bool need = kDec ? (ch == 0 ? p.row_val >= 0 : ch == kCh - 1 ? p.row_lap >= 0 : p.row_dx >= 0)
+          const bool need = kMode == kDecode ? (ch == 0 ? p.row_val >= 0 : ch == kCh - 1 ? p.row_lap >= 0 : p.row_dx >= 0)
                                  : ch >= 1 && (!kFirst || ch == kCh - 1 || p.pde != CROM_PDE_HEAT);
           if (need) {
             float wv[8];
@@ -667,7 +684,7 @@ __device__ __forceinline__ bool forward_tile(Lane& c, const StepParams& p, int j
     const int b = ch * 4 * kSm + s;
     return (pr[b] + pr[b + kSm]) + (pr[b + 2 * kSm] + pr[b + 3 * kSm]);
   };
-  if constexpr (kDec) {  // decode mode: the requested channels of the tile's samples
+  if constexpr (kMode == kDecode) {  // decode mode: the requested channels of the tile's samples
     if (c.gt < ns) {
       const size_t n = (size_t)p.n_samples, j = (size_t)(j0 + c.gt);
       if (p.row_val >= 0) p.dec_out[(size_t)p.row_val * n + j] = gout(0, c.gt) + p.bout;
@@ -709,9 +726,9 @@ __device__ __forceinline__ bool forward_tile(Lane& c, const StepParams& p, int j
 // One tile of kSm samples of one GN iteration k >= 1: forward pass, PDE update /
 // residual, reverse pass, Jacobian projection and this tile's share of J^T J and
 // J^T rho; or, for a line-search trial (kValueOnly), the forward pass and rho^T rho.
-template <int kM, int kSm, bool kLoP, bool kValueOnly = false>
+template <int kM, int kSm, bool kLoP, Mode kMode, bool kValueOnly = false>
 __device__ __forceinline__ bool run_tile(Lane& c, const StepParams& p, int o0, int t, int ns, float alpha, Own& o) {
-  if (!forward_tile<kM, kSm, false, kSm, kLoP>(c, p, o0 + t * kSm, 0, ns, alpha)) return false;
+  if (!forward_tile<kM, kSm, false, kSm, kLoP, kMode>(c, p, o0 + t * kSm, 0, ns, alpha)) return false;
   if constexpr (kValueOnly) {  // line-search trial: only sum_j rho_j^2 is needed
     group_sync(c.g);
 #pragma unroll
@@ -719,7 +736,7 @@ __device__ __forceinline__ bool run_tile(Lane& c, const StepParams& p, int o0, i
       if (o.ea[e] == -3) o.acc[e] += dot_exact<false, false>(c.G->rho, c.G->zero, 1, c.G->rho, c.G->zero, 1, ns);
     return true;
   } else {
-    return reverse_tile<kM, kSm, kSm, kLoP>(c, p, o0 + t * kSm, ns, o);
+    return reverse_tile<kM, kSm, kSm, kLoP, kMode>(c, p, o0 + t * kSm, ns, o);
   }
 }
 
@@ -729,16 +746,16 @@ __device__ __forceinline__ bool run_tile(Lane& c, const StepParams& p, int o0, i
 // the four-channel forward pass needs narrow tiles to fit the 32 hi columns of one
 // N = 64 UMMA, the
 // reverse pass does not.
-template <int kM, bool kLoP, bool kDec = false>
+template <int kM, bool kLoP, Mode kMode>
 __device__ __forceinline__ bool run_pair(Lane& c, const StepParams& p, int o0, int t, int ns, float alpha, Own& o) {
   constexpr int kS0 = tile_s0<kLoP>();
   constexpr int kSS = 2 * kS0;
   const int j0 = o0 + t * kSS;
-  if (!forward_tile<kM, kS0, true, kSS, kLoP, kDec>(c, p, j0, 0, min(ns, kS0), alpha)) return false;
-  const bool rev = !kDec || p.row_dq >= 0;  // decode mode: the reverse pass only for dg/dq
-  if (ns <= kS0) return rev ? reverse_tile<kM, kS0, kSS, kLoP, kDec>(c, p, j0, ns, o) : true;
-  if (!forward_tile<kM, kS0, true, kSS, kLoP, kDec>(c, p, j0 + kS0, kS0, ns - kS0, alpha)) return false;
-  return rev ? reverse_tile<kM, kSS, kSS, kLoP, kDec>(c, p, j0, ns, o) : true;
+  if (!forward_tile<kM, kS0, true, kSS, kLoP, kMode>(c, p, j0, 0, min(ns, kS0), alpha)) return false;
+  const bool rev = kMode != kDecode || p.row_dq >= 0;  // decode mode: the reverse pass only for dg/dq
+  if (ns <= kS0) return rev ? reverse_tile<kM, kS0, kSS, kLoP, kMode>(c, p, j0, ns, o) : true;
+  if (!forward_tile<kM, kS0, true, kSS, kLoP, kMode>(c, p, j0 + kS0, kS0, ns - kS0, alpha)) return false;
+  return rev ? reverse_tile<kM, kSS, kSS, kLoP, kMode>(c, p, j0, ns, o) : true;
 }
 
 
@@ -797,13 +814,164 @@ __device__ __forceinline__ bool decode_chunk(Lane& c, const StepParams& p, int a
     set_layer1<kM>(c, p, G, G->qcur);
     const int M = e - a, nt = (M + 2 * kS0 - 1) / (2 * kS0);
     for (int t = 0; t < nt && ok; ++t)
-      ok = run_pair<kM, kLoP, true>(c, p, a, t, min(2 * kS0, M - t * 2 * kS0), 0.f, o);
+      ok = run_pair<kM, kLoP, kDecode>(c, p, a, t, min(2 * kS0, M - t * 2 * kS0), 0.f, o);
     a = e;
   }
   return ok;
 }
 
-template <int kM, int kS1, bool kLoP, bool kDec = false>
+// ---------------- split mode
+// Tiles of instance i at this iteration; 0 where it takes no part (an invalid range, or a
+// status other than OK after an earlier iteration).
+template <int kSS, Mode kMode>
+__device__ __forceinline__ int iter_tiles(const StepParams& p, int i) {
+  const int o0 = p.off[i], M = p.off[i + 1] - o0;
+  if (kMode == kIterLater) {
+    if (p.status[i] != CROM_OK) return 0;
+  } else if (M < p.r || M > p.max_samples || o0 < 0 || o0 + M > p.n_samples) {
+    return 0;
+  }
+  return (M + kSS - 1) / kSS;
+}
+
+// One Gauss-Newton iteration of all instances: the tiles of all instances in one row are
+// dealt to the groups in equal ranges, each tile's normal-equation terms go to its own row
+// of p.rows, and the group that completes an instance's last tile adds the rows in order
+// of the tiles (the order in which a group that owns the whole instance adds them: the
+// same bits) and solves.  No group waits for another.  A bounded wait that runs out marks
+// the instances of the group's range, which then end as TIMEOUT.
+template <int kM, bool kLoP, Mode kMode>
+__device__ __forceinline__ bool run_iteration(Lane& c, const StepParams& p, Own& own, uint8_t* scratch, int* part, bool ok) {
+  constexpr int kSS = 2 * tile_s0<kLoP>();
+  constexpr int kFail = 1 << 30;
+  Group* G = c.G;
+  const int r = p.r, n_entries = r * (r + 1) / 2 + r, tid = threadIdx.x;
+  // prefix sums of the tile counts, in the operand blocks (not yet in use)
+  int* prefix = reinterpret_cast<int*>(scratch);
+  const int per = (p.n_inst + kThreads - 1) / kThreads, i0 = min(p.n_inst, tid * per), i1 = min(p.n_inst, i0 + per);
+  int sum = 0;
+  for (int i = i0; i < i1; ++i) {
+    const int nt = iter_tiles<kSS, kMode>(p, i);
+    if (kMode == kIterFirst && nt == 0 && blockIdx.x == 0) p.status[i] = CROM_ERR_INVALID_ARG;
+    prefix[i] = sum;
+    sum += nt;
+  }
+  int incl = sum;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, d);
+    if ((tid & 31) >= d) incl += v;
+  }
+  if ((tid & 31) == 31) part[tid >> 5] = incl;
+  __syncthreads();
+  int before = incl - sum, total = 0;
+  for (int w = 0; w < kThreads / 32; ++w) {
+    if (w < tid >> 5) before += part[w];
+    total += part[w];
+  }
+  for (int i = i0; i < i1; ++i) prefix[i] += before;
+  __syncthreads();
+  const int groups = gridDim.x * kGroups, gid = c.g * gridDim.x + blockIdx.x;
+  int a = (int)((long long)total * gid / groups);
+  const int b = (int)((long long)total * (gid + 1) / groups);
+  int inst = 0, base = 0;
+  if (a < b) {  // the last instance with prefix <= a (those without tiles share a prefix)
+    int lo = 0, hi = p.n_inst;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (prefix[mid] <= a) lo = mid;
+      else hi = mid;
+    }
+    inst = lo;
+    base = prefix[lo];
+  }
+  __syncthreads();  // the operand blocks are free again
+  for (; a < b; ++inst) {
+    const int nt = iter_tiles<kSS, kMode>(p, inst);
+    if (nt == 0) continue;
+    const int e = min(b, base + nt), o0 = p.off[inst], M = p.off[inst + 1] - o0;
+    if (base + nt > p.rows_cap) {  // only offsets that decrease give more tiles than the samples hold
+      if (a == base && c.gt == 0) p.status[inst] = CROM_ERR_INVALID_ARG;
+      a = e;
+      base += nt;
+      continue;
+    }
+    group_sync(c.g);  // the previous range's group state is no longer read
+    if (c.gt < r) {
+      const double v = p.q[(size_t)inst * r + c.gt];
+      G->qn[c.gt] = kMode == kIterFirst ? v : p.qbase[(size_t)inst * r + c.gt];
+      G->qcur[c.gt] = v;
+    }
+    group_sync(c.g);
+    if (ok) {
+      const float alpha = p.coef_per_sample ? 0.f : p.alpha[inst];
+      set_layer1<kM>(c, p, G, G->qcur);
+      for (int t = a - base; t < e - base && ok; ++t) {
+        own.row = p.rows + (size_t)(base + t) * n_entries;
+        const int ns = min(kSS, M - t * kSS);
+        if constexpr (kMode == kIterFirst) ok = run_pair<kM, kLoP, kMode>(c, p, o0, t, ns, alpha, own);
+        else ok = run_tile<kM, kSS, kLoP, kMode>(c, p, o0, t, ns, alpha, own);
+      }
+    }
+    group_sync(c.g);  // every thread's terms are written
+    if (c.gt == 0) {
+      __threadfence();
+      if (!ok) atomicOr(&p.counters[inst], kFail);
+      const int old = atomicAdd(&p.counters[inst], e - a);
+      __threadfence();
+      G->s_idx = (old & (kFail - 1)) + (e - a) == nt ? ((old & kFail) ? 2 : 1) : 0;
+    }
+    group_sync(c.g);
+    const int last = G->s_idx;
+    if (last) {
+      const int R = r + 1;
+      if (last == 1) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const int ea = own.ea[k], eb = own.eb[k];
+          if (ea < 0) continue;
+          const double* x = p.rows + (size_t)base * n_entries + c.gt + k * kGT;
+          double acc = 0.0;
+          for (int t0 = 0; t0 < nt; t0 += 16) {  // loads ahead of the additions
+            double v[16];
+#pragma unroll
+            for (int t = 0; t < 16; ++t)
+              if (t0 + t < nt) v[t] = __ldcg(x + (size_t)(t0 + t) * n_entries);
+#pragma unroll
+            for (int t = 0; t < 16; ++t)
+              if (t0 + t < nt) acc += v[t];
+          }
+          if (eb >= 0) {
+            G->amat[ea * R + eb] = acc;
+            G->amat[eb * R + ea] = acc;
+          } else {
+            G->amat[ea * R + r] = -acc;
+          }
+        }
+      }
+      group_sync(c.g);
+      if (c.gw == 0) {
+        int st = CROM_ERR_TIMEOUT;
+        if (last == 1) {
+          st = chol_solve_warp(G->amat, G->invd, r, c.gt);
+          if (st == CROM_OK && c.gt < r) {
+            if (kMode == kIterFirst) p.qbase[(size_t)inst * r + c.gt] = G->qn[c.gt];
+            p.q[(size_t)inst * r + c.gt] = G->qcur[c.gt] + G->amat[c.gt * R + r];
+          }
+        }
+        if (c.gt == 0) {
+          p.status[inst] = st;
+          p.counters[inst] = 0;
+        }
+      }
+    }
+    a = e;
+    base += nt;
+  }
+  return ok;
+}
+
+template <int kM, int kS1, bool kLoP, Mode kMode = kStep>
 __global__ void __launch_bounds__(kThreads, 1) step_tc_kernel(StepParams p) {
   constexpr int kS0 = tile_s0<kLoP>();
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -891,12 +1059,16 @@ __global__ void __launch_bounds__(kThreads, 1) step_tc_kernel(StepParams p) {
     own.eb[e] = eb;
   }
 
-  while (ok) {
+  if constexpr (kMode >= kIterFirst) {
+    if (kMode == kIterFirst && blockIdx.x == 0 && tid == 0) p.queue[1] = 0;  // the timeout flag
+    ok = run_iteration<kM, kLoP, kMode>(c, p, own, Hbase, S->part, ok);
+  }
+  while (kMode < kIterFirst && ok) {
     group_sync(c.g);  // everyone is done with the previous instance's group state
     if (c.gt == 0) G->s_idx = atomicAdd(&p.queue[0], 1);
     group_sync(c.g);
     const int idx = G->s_idx;
-    if constexpr (kDec) {  // decode mode: work item idx is a chunk of kDecChunk points
+    if constexpr (kMode == kDecode) {  // decode mode: work item idx is a chunk of kDecChunk points
       const long a0 = (long)idx * kDecChunk;
       if (a0 >= p.n_samples) break;
       ok = decode_chunk<kM, kLoP>(c, p, (int)a0, (int)min(a0 + kDecChunk, (long)p.n_samples), own);
@@ -925,11 +1097,11 @@ __global__ void __launch_bounds__(kThreads, 1) step_tc_kernel(StepParams p) {
       if (it == 0) {
         const int nt = (M + 2 * kS0 - 1) / (2 * kS0);
         for (int t = 0; t < nt && ok; ++t)
-          ok = run_pair<kM, kLoP>(c, p, o0, t, min(2 * kS0, M - t * 2 * kS0), alpha, own);
+          ok = run_pair<kM, kLoP, kStep>(c, p, o0, t, min(2 * kS0, M - t * 2 * kS0), alpha, own);
       } else {
         const int nt = (M + kS1 - 1) / kS1;
         for (int t = 0; t < nt && ok; ++t)
-          ok = run_tile<kM, kS1, kLoP>(c, p, o0, t, min(kS1, M - t * kS1), alpha, own);
+          ok = run_tile<kM, kS1, kLoP, kStep>(c, p, o0, t, min(kS1, M - t * kS1), alpha, own);
       }
       if (!ok) break;
       const int R = r + 1;
@@ -977,7 +1149,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_tc_kernel(StepParams p) {
           own.acc[0] = own.acc[1] = 0.0;
           const int nt = (M + kS1 - 1) / kS1;
           for (int t = 0; t < nt && ok; ++t)
-            ok = run_tile<kM, kS1, kLoP, true>(c, p, o0, t, min(kS1, M - t * kS1), alpha, own);
+            ok = run_tile<kM, kS1, kLoP, kStep, true>(c, p, o0, t, min(kS1, M - t * kS1), alpha, own);
           if (!ok) break;
 #pragma unroll
           for (int e = 0; e < 2; ++e)
@@ -1055,6 +1227,37 @@ size_t tc_step_smem_bytes(int img_bytes) {
          kGroups * sizeof(Group);
 }
 
+namespace {
+// Grows a scratch array of the context to n elements.
+template <typename T>
+cudaError_t grow(crom_ctx* ctx, T** buf, size_t* cap, size_t n) {
+  if (n <= *cap) return cudaSuccess;
+  if (*buf) cudaFree(*buf);
+  ++ctx->scratch_gen;
+  *buf = nullptr;
+  *cap = 0;
+  const cudaError_t e = cudaMalloc(buf, n * sizeof(T));
+  if (e == cudaSuccess) *cap = n;
+  return e;
+}
+// Whether a step's iterations are launches of their own with the tiles dealt to all
+// groups, or one launch whose groups own whole instances.  In tiles per group: the split
+// iterations take about T / G (T tiles on G groups) and the cost of one tile more; the
+// groups of the whole form wait for the largest instance, and with more instances than
+// groups for a second round of equal ones.  Measured, two iterations, F16X2, whole against
+// split: 1 x 200 samples 342 / 67 us, 8 x 4096 8899 / 240 us, 450 x (32..512) 1140 / 603 us,
+// 700 x 256 1084 / 785 us; but 608 x 256 611 / 637 us and 1024 x (32..512) 1156 / 1213 us.
+// Far above one instance per group only the caller's bound on |M_i| could ask for it.
+bool split_wanted(int n_inst, int n_samples, int max_samples, int tile, int num_sms) {
+  const double G = kGroups * num_sms;
+  if (n_inst > 1.25 * G) return false;
+  const double mean = (double)n_samples / n_inst / tile, T = (mean + 0.5) * n_inst;
+  const double largest = ceil((double)std::min(max_samples, n_samples) / tile);
+  const double whole = largest <= 1.25 * mean ? std::max(largest, ceil(n_inst / G) * mean) : largest;
+  return whole >= ceil(T / G) + 1.0 && whole >= 1.15 * T / G;
+}
+}  // namespace
+
 cudaError_t launch_step_tc(crom_ctx* ctx, const crom_step_desc* step, int lo_parts, int n_inst, double* q,
                            const float* alpha, const float* vel, const int* s_off, const float* samples,
                            int n_samples, int max_samples, int* status, cudaStream_t s) {
@@ -1076,8 +1279,24 @@ cudaError_t launch_step_tc(crom_ctx* ctx, const crom_step_desc* step, int lo_par
     if (e != cudaSuccess) return e;
     ctx->targets_cap = n_samples;
   }
-  order_kernel<<<1, 1024, 0, s>>>(s_off, n_inst, ctx->order, status, ctx->queue);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  constexpr int kLarge = kTcTileS1Large, kSmall = kTcTileS1Small;
+  const bool small_tiles = ctx->tc_tile_s1 == kSmall;
+  // Split mode: see split_wanted.  Its tile rows are sized for every instance's ragged
+  // last tile.
+  const int tile = lo_parts ? kLarge : 2 * kLarge, n_entries = ctx->desc.r * (ctx->desc.r + 3) / 2;
+  const bool split = step->line_search == 0 && !small_tiles && split_wanted(n_inst, n_samples, max_samples, tile, ctx->num_sms);
+  if (split) {
+    if ((e = grow(ctx, &ctx->partials, &ctx->partials_cap, ((size_t)n_samples / tile + n_inst) * n_entries)) != cudaSuccess ||
+        (e = grow(ctx, &ctx->qbase, &ctx->qbase_cap, (size_t)n_inst * ctx->desc.r)) != cudaSuccess)
+      return e;
+    const size_t cap = ctx->counters_cap;
+    if ((e = grow(ctx, &ctx->counters, &ctx->counters_cap, (size_t)n_inst)) != cudaSuccess) return e;
+    if (ctx->counters_cap != cap && (e = cudaMemset(ctx->counters, 0, (size_t)n_inst * sizeof(int))) != cudaSuccess) return e;
+  } else {
+    order_kernel<<<1, 1024, 0, s>>>(s_off, n_inst, ctx->order, status, ctx->queue);
+    e = cudaGetLastError();
+  }
   if (e != cudaSuccess) return e;
   StepParams p{};
   p.img = ctx->w.tc_img;
@@ -1111,16 +1330,33 @@ cudaError_t launch_step_tc(crom_ctx* ctx, const crom_step_desc* step, int lo_par
   p.order = ctx->order;
   p.queue = ctx->queue;
   p.df = ctx->targets;
+  p.qbase = ctx->qbase;
+  p.rows = ctx->partials;
+  p.rows_cap = n_samples / tile + n_inst;
+  p.counters = ctx->counters;
   const size_t smem = tc_step_smem_bytes(p.img_bytes);
-  const int grid = std::min((n_inst + kGroups - 1) / kGroups, ctx->num_sms);
+  const int grid = split ? (int)std::min<long long>((long long)n_samples / tile + n_inst, ctx->num_sms)
+                         : std::min((n_inst + kGroups - 1) / kGroups, ctx->num_sms);
   auto launch = [&](auto kernel) -> cudaError_t {
     cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     kernel<<<grid, kThreads, smem, s>>>(p);
     return cudaGetLastError();
   };
-  constexpr int kLarge = kTcTileS1Large, kSmall = kTcTileS1Small;
-  const bool small_tiles = ctx->tc_tile_s1 == kSmall;
+  if (split) {
+    const bool two = ctx->desc.m == 2;
+    for (int it = 0; it < step->gn_iters && e == cudaSuccess; ++it) {
+      if (lo_parts)
+        e = it == 0 ? (two ? launch(step_tc_kernel<2, kLarge, true, kIterFirst>) : launch(step_tc_kernel<1, kLarge, true, kIterFirst>))
+                    : (two ? launch(step_tc_kernel<2, kLarge, true, kIterLater>) : launch(step_tc_kernel<1, kLarge, true, kIterLater>));
+      else
+        e = it == 0 ? (two ? launch(step_tc_kernel<2, 2 * kLarge, false, kIterFirst>)
+                           : launch(step_tc_kernel<1, 2 * kLarge, false, kIterFirst>))
+                    : (two ? launch(step_tc_kernel<2, 2 * kLarge, false, kIterLater>)
+                           : launch(step_tc_kernel<1, 2 * kLarge, false, kIterLater>));
+    }
+    return e;
+  }
   if (lo_parts) {
     if (ctx->desc.m == 2)
       return small_tiles ? launch(step_tc_kernel<2, kSmall, true>) : launch(step_tc_kernel<2, kLarge, true>);
@@ -1181,9 +1417,9 @@ cudaError_t launch_decode_tc(crom_ctx* ctx, int lo_parts, int n_inst, const doub
   // the later-iteration tile size is not used in decode mode: the default instantiations
   constexpr int kLarge = kTcTileS1Large;
   if (lo_parts)
-    return m == 2 ? launch(step_tc_kernel<2, kLarge, true, true>) : launch(step_tc_kernel<1, kLarge, true, true>);
-  return m == 2 ? launch(step_tc_kernel<2, 2 * kLarge, false, true>)
-                : launch(step_tc_kernel<1, 2 * kLarge, false, true>);
+    return m == 2 ? launch(step_tc_kernel<2, kLarge, true, kDecode>) : launch(step_tc_kernel<1, kLarge, true, kDecode>);
+  return m == 2 ? launch(step_tc_kernel<2, 2 * kLarge, false, kDecode>)
+                : launch(step_tc_kernel<1, 2 * kLarge, false, kDecode>);
 }
 
 }  // namespace crom
