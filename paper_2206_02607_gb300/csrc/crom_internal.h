@@ -149,7 +149,8 @@ struct crom_trainer {
   std::vector<float*> Z, H;  // per hidden layer: [B*S][width]
   float *delta = nullptr, *delta2 = nullptr, *din = nullptr, *dq = nullptr;
   float* split = nullptr;  // split-K partial sums of weight gradients
-  float *edh = nullptr, *edx = nullptr, *ed1 = nullptr;
+  float* ed1 = nullptr;
+  double* conv_part = nullptr;  // convolution gradients' partial sums
   double* partial = nullptr;
   double* loss_dev = nullptr;
   double* red = nullptr;  // partial sums of the deterministic column / convolution reductions
