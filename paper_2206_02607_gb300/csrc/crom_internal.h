@@ -121,10 +121,10 @@ struct TrainerTc {
   uint16_t* wh = nullptr;   // bf16 hidden matrices W_1..W_{L-1}, [w][w] each
   std::vector<uint16_t*> H; // bf16 activations of the hidden layers, [B*S][w] each
   uint16_t *d0 = nullptr, *d1 = nullptr;  // bf16 deltas [B*S][w]
-  float *colpart = nullptr, *colpart2 = nullptr, *rowpart = nullptr;  // per-32-row partial sums
-  float* resid = nullptr;   // [B*S]: g - f per point (FP32)
-  float* colmid = nullptr;  // first level of the column-sum reduction
-  float* split = nullptr;   // split-K partials of the weight gradients
+  // partial sums of a step, reduced together at its end: per 32 rows the columns' (set 0:
+  // dw_out, set h: db_h) and the rows'; the first level of the former; the weight
+  // gradients' K ranges
+  float *colpart = nullptr, *rowpart = nullptr, *colmid = nullptr, *split = nullptr;
   float* xin = nullptr;     // [B*S][m]: the sampled points' coordinates
   float* c0 = nullptr;      // [B][w]: b_0 + W_0q q_b, the latent part of layer 0 per snapshot
   float* part0 = nullptr;   // [B][chunks][w][1 + m]: row-chunk moments of delta_0
@@ -243,8 +243,9 @@ enum GemmEpi {
   kGemmEpiF32 = 0,        // out_f32[split][m][n] = D (K split into `splits` ranges)
   kGemmEpiBiasElu = 1,    // out_bf16[m][n] = ELU(D + bias[n])
   kGemmEpiTimesEluD = 2,  // out_bf16[m][n] = D * s'(z), s' from hprev[m][n] = h = ELU(z); colpart = column sums
-  kGemmEpiOut = 3         // last hidden layer: out_bf16 = h_L = ELU(D + bias); per row the residual
-                          // resid[m] = wout . h_L + *bout - target[m] (FP32 from the FP32 h_L)
+  kGemmEpiOut = 3         // last hidden layer: h_L = ELU(D + bias), per row the residual r = wout . h_L +
+                          // *bout - target[m] (FP32 from the FP32 h_L); out_bf16 = delta_L = 2 r inv_count
+                          // wout s'(z) from bf16 h_L, with its column and row sums
 };
 struct TcGemm {
   int M = 0, N = 0, K = 0;
@@ -261,11 +262,13 @@ struct TcGemm {
   uint16_t* out_bf16 = nullptr;
   const float* bias = nullptr;
   const uint16_t* hprev = nullptr;
-  float* colpart = nullptr;  // [ceil(M / 128) * 4][N]: per-warp column sums (32 rows each)
+  float* colpart = nullptr;   // [ceil(M / 128) * 4][N]: per-warp column sums (32 rows each), or null
+  float* colpart2 = nullptr;  // output layer: the same for 2 r inv_count h_L
+  float* rowpart = nullptr;   // output layer: [ceil(M / 128) * 4][2]: sums of r^2 and of 2 r inv_count
   const float* wout = nullptr;
   const float* bout = nullptr;  // device scalar
   const float* target = nullptr;
-  float* resid = nullptr;  // [M]
+  float inv_count = 0.f;
 };
 bool tc_gemm_supported(int n);
 cudaError_t tc_gemm(const TcGemm& g, int num_sms, int* flag, cudaStream_t s);

@@ -2,18 +2,18 @@
 // App. D): D[m][n] = sum_k A(m, k) B(n, k) with FP32 accumulation in tensor memory
 // and the training pass's elementwise work fused into the epilogue.
 //
-// Persistent, one CTA per SM, 320 threads in warp roles:
+// Persistent, one CTA per SM, 320 or 576 threads in warp roles:
 //   warp 0   TMA producer: one elected lane loads the A and B boxes of each 64-wide
 //            K block (cp.async.bulk.tensor, 128-byte swizzle) into a 3-stage ring;
 //   warp 1   MMA issuer: four UMMAs (M = 128, N = BN, K = 16) per K block into one of
 //            two tensor-memory accumulators, commits free the ring stage and, after
 //            the tile's last block, hand the accumulator to the epilogue;
-//   warps 2-9 epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (one tile row per
-//            thread) and one half of the BN columns (warps 2-5 the first, 6-9 the
-//            second), applies the fused operation, frees the accumulator; bf16 rows
+//   warps 2.. epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (one tile row per
+//            thread) and one part of the BN columns (a half or a quarter: warps 2-5 the
+//            first, 6-9 the second, ..), applies the fused operation, frees the accumulator; bf16 rows
 //            go through a per-warp shared-memory staging area so that global loads
-//            and stores move whole half rows (coalesced).  Two warps per SM
-//            sub-partition hide each other's load, shuffle and exp latencies.
+//            and stores move whole parts of rows (coalesced).  Two or four warps per
+//            SM sub-partition hide each other's load, shuffle and exp latencies.
 // With two accumulators the epilogue of one tile overlaps the MMAs of the next.
 // Operands: A(m, k) K-major (A[m * lda + k]) or MN-major (A[k * lda + m]); B(n, k)
 // likewise; both are read through tensor maps whose boxes land in shared memory in
@@ -26,6 +26,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "crom_internal.h"
 #include "tc_common.cuh"
@@ -36,8 +37,12 @@ namespace {
 using namespace tc;
 
 constexpr int kBM = 128, kBK = 64, kStages = 3;
-constexpr int kEpiWarps = 8;
-constexpr int kGemmThreads = 64 + 32 * kEpiWarps;
+// Column parts of a tile's epilogue, a warp of each for every 32 rows.  Two hold the issue
+// slots at 40 %, waiting on tensor memory, shuffles and the staging rows; four hide that
+// (the s' epilogue 88 -> 80 us at 2^18 rows of 256, bias + ELU 52 -> 50 us) where the parts
+// keep 32 columns.  The output layer's sum over the columns is one chain per half.
+template <int kBN, int kEpi>
+constexpr int kParts = kBN >= 128 && (kEpi == kGemmEpiTimesEluD || kEpi == kGemmEpiBiasElu) ? 4 : 2;
 constexpr uint32_t kWait = 1u << 26;
 
 struct Args {
@@ -50,11 +55,13 @@ struct Args {
   uint16_t* out_bf16;
   const float* bias;
   const uint16_t* hprev;
-  float* colpart;   // [tiles_m * 4][N]
+  float* colpart;   // [tiles_m * 4][N], or null
+  float* colpart2;  // output-layer epilogue: the same for dL/dg h
+  float* rowpart;   // output-layer epilogue: [tiles_m * 4][2]
   const float* wout;
   const float* bout;
   const float* target;
-  float* resid;     // [M]: g - target per row (output-layer epilogue)
+  float inv_count;
   int* flag;
 };
 
@@ -198,6 +205,63 @@ struct Staging {
     }
     __syncwarp();
   }
+  // The output layer's reverse pass on the staged rows h_L (bf16), lane l their columns
+  // l kC .. (kC = kW / 32): with r the row's residual (lane i holds row i's), dL/dg =
+  // 2 r inv_count and delta_L = dL/dg w_out s'(z), s' = 1 where h > 0, else h + 1, in place
+  // of h.  The part's column sums of delta (db_L) and of dL/dg h (dw_out) and its row sums of
+  // r^2 and dL/dg, each in row order.  As a kernel of its own over h_L written to memory it
+  // took 50 us after a GEMM of 66 us (2^18 rows of 256); the GEMM with it, 99 us.
+  __device__ __forceinline__ void out_delta(int lane, int cb, int row0, int M, float r, float inv_count,
+                                            const float* wout, long part, int ldc, bool rows, float* colpart,
+                                            float* colpart2, float* rowpart) const {
+    constexpr int kC = kW / 32;
+    float wo[kC], cs[kC], cs2[kC];
+#pragma unroll
+    for (int k = 0; k < kC; ++k) {
+      wo[k] = wout[lane * kC + k];
+      cs[k] = 0.f;
+      cs2[k] = 0.f;
+    }
+    float rr = 0.f, dgs = 0.f;
+    union Vec {
+      uint16_t u[kC];
+      typename std::conditional<kC == 4, uint2, typename std::conditional<kC == 2, uint32_t, uint16_t>::type>::type v;
+    };
+    constexpr int kAhead = 8;  // rows read before they are worked on
+#pragma unroll 1
+    for (int i0 = 0; i0 < 32; i0 += kAhead) {
+      Vec x[kAhead];
+#pragma unroll
+      for (int j = 0; j < kAhead; ++j)
+        x[j].v = *reinterpret_cast<const decltype(x[j].v)*>(base + (i0 + j) * kSt + lane * kC);
+#pragma unroll
+      for (int j = 0; j < kAhead; ++j) {
+        const float res = __shfl_sync(0xffffffffu, r, i0 + j);
+        const float dg = 2.f * res * inv_count;
+        const bool in = row0 + i0 + j < M;
+#pragma unroll
+        for (int k = 0; k < kC; ++k) {
+          const float h = in ? __uint_as_float((uint32_t)x[j].u[k] << 16) : 0.f;
+          const float d = dg * wo[k] * (h > 0.f ? 1.f : h + 1.f);
+          cs[k] += d;
+          cs2[k] = fmaf(dg, h, cs2[k]);
+          x[j].u[k] = to_bf16(d);
+        }
+        *reinterpret_cast<decltype(x[j].v)*>(base + (i0 + j) * kSt + lane * kC) = x[j].v;
+        rr = fmaf(res, res, rr);
+        dgs += dg;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kC; ++k) {
+      colpart[part * ldc + cb + lane * kC + k] = cs[k];
+      colpart2[part * ldc + cb + lane * kC + k] = cs2[k];
+    }
+    if (rows && lane == 0) {
+      rowpart[2 * part] = rr;
+      rowpart[2 * part + 1] = dgs;
+    }
+  }
   // load_rows in two halves: fetch_rows issues the global loads into registers (the
   // loads stay in flight while the caller does other work), put_rows writes them to
   // the staging rows
@@ -225,13 +289,14 @@ struct Staging {
 };
 
 template <int kBN, int kEpi>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(64 + 128 * kParts<kBN, kEpi>, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, Args g) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   constexpr uint32_t kABytes = kBM * kBK * 2, kBBytes = kBN * kBK * 2, kStageBytes = kABytes + kBBytes;
-  constexpr int kHalf = kBN / 2;  // columns per epilogue warp
-  constexpr size_t kStgBytes = (size_t)kEpiWarps * 32 * Staging<kHalf>::kSt * 2;
+  constexpr int kEpiWarps = 4 * kParts<kBN, kEpi>;
+  constexpr int kCols = kBN / kParts<kBN, kEpi>;  // columns per epilogue warp
+  constexpr size_t kStgBytes = (size_t)kEpiWarps * 32 * Staging<kCols>::kSt * 2;
   Bars* bars = reinterpret_cast<Bars*>(sm + kStages * kStageBytes + kStgBytes);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
@@ -333,8 +398,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     // ------------------------------------------------ epilogue
     const int ew = warp - 2;
     const int q = warp & 3;                 // TMEM lane quadrant of this warp
-    const int half = ew >> 2, cb = half * kHalf;  // its column half
-    const Staging<kHalf> stg{reinterpret_cast<uint16_t*>(sm + kStages * kStageBytes) + ew * 32 * Staging<kHalf>::kSt};
+    const int half = ew >> 2, cb = half * kCols;  // its column part
+    const Staging<kCols> stg{reinterpret_cast<uint16_t*>(sm + kStages * kStageBytes) + ew * 32 * Staging<kCols>::kSt};
     uint32_t tphase[2] = {0, 0};
     int local = 0;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++local) {
@@ -351,7 +416,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       tc_fence_after();
       const uint32_t ta = tb + (uint32_t)acc * kBN + (uint32_t)cb + ((uint32_t)(q * 32) << 16);
       float gval = 0.f;
-      constexpr int kCh = kHalf / 32;
+      constexpr int kCh = kCols / 32;
       const float* sbias = bars->bias + cb;
       const float* swout = bars->wout + cb;
       if (kEpi == kGemmEpiOut) {
@@ -385,8 +450,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 #pragma unroll
           for (int j = 0; j < 32; ++j) v[j] = in ? v[j] * elud_from_h(hp[j]) : 0.f;
           stg.put32(lane, c0, v);                    // in place of the h values just read
-          const float cs = warp_colsum32(v, lane);  // column sums of delta over this warp's rows
-          g.colpart[(long)(mt * 4 + q) * g.N + col + lane] = cs;
+          if (g.colpart) {  // column sums of delta over this warp's rows
+            const float cs = warp_colsum32(v, lane);
+            g.colpart[(long)(mt * 4 + q) * g.N + col + lane] = cs;
+          }
         }
       });
       }
@@ -398,19 +465,21 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       if (kEpi == kGemmEpiTimesEluD) {
         // the next tile's h_{l-1} rows are loaded while this tile's delta rows are stored
         const int tn = t + gridDim.x;
-        uint4 R[Staging<kHalf>::kFetch];
+        uint4 R[Staging<kCols>::kFetch];
         if (tn < tiles) stg.fetch_rows(g.hprev, g.ldo, (tn % g.tiles_m) * kBM + q * 32, cb, g.M, lane, R);
         stg.store_rows(g.out_bf16, g.ldo, row0, cb, g.M, lane);
         if (tn < tiles) stg.put_rows(lane, R);
       }
       if (kEpi == kGemmEpiOut) {
-        stg.store_rows(g.out_bf16, g.ldo, row0, cb, g.M, lane);
         // the two column halves' partial sums meet in shared memory, added in a fixed
-        // order; the residual g - target of each row
+        // order: the residual g - target of each row
         bars->gpart[local & 1][half][q][lane] = gval;
         asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory");  // the two warps of quadrant q
         gval = bars->gpart[local & 1][0][q][lane] + bars->gpart[local & 1][1][q][lane];
-        if (half == 0 && in) g.resid[row] = gval + __ldg(g.bout) - __ldg(g.target + row);
+        const float res = in ? gval + __ldg(g.bout) - __ldg(g.target + row) : 0.f;
+        stg.out_delta(lane, cb, row0, g.M, res, g.inv_count, swout, (long)(mt * 4 + q), g.N, half == 0, g.colpart,
+                      g.colpart2, g.rowpart);
+        stg.store_rows(g.out_bf16, g.ldo, row0, cb, g.M, lane);
       }
     }
   }
@@ -459,11 +528,11 @@ bool make_map(CUtensorMap* m, const void* base, long inner, long outer, long ld,
 template <int kBN, int kEpi>
 cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tbm, const Args& a, int grid, cudaStream_t s) {
   const size_t smem = 1024 + (size_t)kStages * (kBM * kBK * 2 + kBN * kBK * 2) +
-                      (size_t)kEpiWarps * 32 * Staging<kBN / 2>::kSt * 2 + sizeof(Bars);
+                      (size_t)kBN * 128 * 2 + 4 * kParts<kBN, kEpi> * 32 * 16 + sizeof(Bars);
   auto k = gemm_tc_kernel<kBN, kEpi>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k<<<grid, kGemmThreads, smem, s>>>(ta, tbm, a);
+  k<<<grid, 64 + 128 * kParts<kBN, kEpi>, smem, s>>>(ta, tbm, a);
   return cudaGetLastError();
 }
 
@@ -509,7 +578,9 @@ cudaError_t tc_gemm(const TcGemm& p, int num_sms, int* flag, cudaStream_t s) {
   a.wout = p.wout;
   a.bout = p.bout;
   a.target = p.target;
-  a.resid = p.resid;
+  a.colpart2 = p.colpart2;
+  a.rowpart = p.rowpart;
+  a.inv_count = p.inv_count;
   a.flag = flag;
   const long tiles = (long)a.tiles_m * a.splits;
   const int grid = (int)std::min<long>(tiles, num_sms);

@@ -9,10 +9,9 @@
 //   forward:  H[0] on the CUDA cores: the latent part W_0q q_b + b_0 is one vector per
 //             snapshot, so a point costs m FMAs per unit;
 //             H[h] = ELU(H[h-1] W_h^T + b_h) by the GEMM's bias + ELU epilogue;
-//             the last layer's epilogue also forms g (FP32, from the FP32 h) and the
-//             residual g - f; a row kernel then forms dL/dg, delta[L-1] =
-//             dL/dg w_out s'(z_{L-1}) and the column sums that give the gradients of
-//             w_out, b_out and b_{L-1};
+//             the last layer's epilogue also forms g (FP32, from the FP32 h), the
+//             residual g - f, dL/dg, delta[L-1] = dL/dg w_out s'(z_{L-1}) and the column
+//             sums that give the gradients of w_out, b_out and b_{L-1};
 //   backward: for h = L-1 .. 1: dW_h = delta[h]^T H[h-1] (K = B*S, split over CTAs,
 //             the splits added in a fixed order) and delta[h-1] = (delta[h] W_h) s'(z_{h-1})
 //             with its column sums (db_{h-1}); then one pass over delta[0] forms, per
@@ -256,100 +255,52 @@ __global__ void layer0_grad_kernel(const float* snap, const float* q, const floa
   }
 }
 
-// The output layer's backward from h_L (bf16 rows of kW) and the residuals r = g - f
-// (FP32, from the GEMM epilogue that formed g from the FP32 h_L): per row
-// dL/dg = 2 r / N and delta_L[n][u] = dL/dg w_out[u] s'(z_u), s'(z) = 1 where h > 0,
-// else h + 1.  Warp p handles rows 32 p .. 32 p + 31 (one part), lane l columns
-// l kPer .. (kPer = kW / 32), four rows' loads in flight; per part the column sums of
-// delta (db_L) and of dL/dg h (dw_out) and the row sums of r^2 and dL/dg, each in
-// row order.
-constexpr int kOutWarps = 8;
-template <int kW>
-__global__ void out_delta_kernel(const uint16_t* H, const float* resid, const float* wout, long N, long nparts,
-                                 float inv_count, uint16_t* delta, float* colpart, float* colpart2, float* rowpart) {
-  constexpr int kPer = kW / 32;  // 2, 4 or 8 bf16 per lane
-  typedef typename std::conditional<kPer == 8, uint4, typename std::conditional<kPer == 4, uint2, uint32_t>::type>::type
-      Vec;
-  const long part = (long)blockIdx.x * kOutWarps + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  const long r0 = part * 32;
-  if (part >= nparts) return;  // whole warps; parts past N write zero sums
-  float wo[kPer], cs[kPer], cs2[kPer];
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    wo[k] = wout[lane * kPer + k];
-    cs[k] = 0.f;
-    cs2[k] = 0.f;
-  }
-  float rr = 0.f, dgs = 0.f;
-  for (int i0 = 0; i0 < 32; i0 += 4) {
-    Vec hv[4];
-    float res[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const long n = r0 + i0 + j;
-      const bool in = n < N;
-      hv[j] = in ? *reinterpret_cast<const Vec*>(H + n * kW + lane * kPer) : Vec{};
-      res[j] = in ? resid[n] : 0.f;
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const long n = r0 + i0 + j;
-      const uint32_t* hw = reinterpret_cast<const uint32_t*>(&hv[j]);
-      const float dg = 2.f * res[j] * inv_count;
-      uint32_t dw[kPer / 2];
-#pragma unroll
-      for (int k = 0; k < kPer / 2; ++k) {
-        const float h0 = bf16_val((uint16_t)(hw[k] & 0xffffu)), h1 = bf16_val((uint16_t)(hw[k] >> 16));
-        const float d0 = dg * wo[2 * k] * (h0 > 0.f ? 1.f : h0 + 1.f);
-        const float d1 = dg * wo[2 * k + 1] * (h1 > 0.f ? 1.f : h1 + 1.f);
-        cs[2 * k] += d0;
-        cs[2 * k + 1] += d1;
-        cs2[2 * k] = fmaf(dg, h0, cs2[2 * k]);
-        cs2[2 * k + 1] = fmaf(dg, h1, cs2[2 * k + 1]);
-        dw[k] = (uint32_t)bf16_bits(d0) | ((uint32_t)bf16_bits(d1) << 16);
-      }
-      if (n < N) *reinterpret_cast<Vec*>(delta + n * kW + lane * kPer) = *reinterpret_cast<const Vec*>(dw);
-      rr = fmaf(res[j], res[j], rr);
-      dgs += dg;
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    colpart[part * kW + lane * kPer + k] = cs[k];
-    colpart2[part * kW + lane * kPer + k] = cs2[k];
-  }
-  if (lane == 0) {
-    rowpart[2 * part] = rr;
-    rowpart[2 * part + 1] = dgs;
-  }
-}
-
-// out[e] = sum_p part[p * stride + e], in order of p (compensated).  Eight loads are
-// issued before their additions, so that their latencies overlap.
-__global__ void sum_parts_kernel(const float* part, int nparts, long stride, long n, float* out) {
-  const long e = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (e >= n) return;
-  CSum s;
-  int p = 0;
-  for (; p + 8 <= nparts; p += 8) {
-    float v[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = __ldg(part + (long)(p + k) * stride + e);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) s.add(v[k]);
-  }
-  for (; p < nparts; ++p) s.add(part[(long)p * stride + e]);
-  out[e] = s.value();
-}
-
-// Column sums of part [nparts][cols] in a fixed order, first level: block (x, y)
-// adds parts y * kColPer .. of columns 32 x .. (32 columns x 8 part lanes, the lanes
-// combined in order) into mid[y][col].  The second level adds mid's rows in order
-// (sum_parts_kernel).
+// The step's remaining sums, all at its end in two launches (a pair per layer and one for
+// the loss took 108 us of launches with one to 256 blocks; these 32 us).
+// First level: set z of the column sums, block (x, y) adds parts y kColPer .. of columns
+// 32 x .. (32 columns x 8 part lanes, the lanes combined in order) into mid[z][y][col].
+// The blocks of z = n_sets reduce the rows' sums, of r^2 to the loss and of dL/dg to db_out:
+// 1024 contiguous ranges of parts (compensated), then a fixed tree in FP64.
 constexpr int kColPer = 128;
-__global__ void colsum_level1_kernel(const float* part, int nparts, int cols, float* mid) {
+__global__ void __launch_bounds__(256) sums_level1_kernel(const float* part, const float* rowpart, int nparts, int cols,
+                                                          int n_sets, double inv_count, float* mid, double* loss,
+                                                          float* gbout) {
+  if ((int)blockIdx.z == n_sets) {
+    if (blockIdx.x + blockIdx.y > 0) return;
+    constexpr int kT = 256, kRanges = 4;
+    __shared__ double red[2][kT];
+    const int tid = threadIdx.y * 32 + threadIdx.x, per = (nparts + kT * kRanges - 1) / (kT * kRanges);
+    double ta = 0.0, tb = 0.0;
+    for (int k = 0; k < kRanges; ++k) {
+      CSum a, b;
+      const int p0 = (tid * kRanges + k) * per, p1 = min(nparts, p0 + per);
+#pragma unroll 8
+      for (int p = p0; p < p1; ++p) {
+        const float2 v = __ldg(reinterpret_cast<const float2*>(rowpart) + p);
+        a.add(v.x);
+        b.add(v.y);
+      }
+      ta += (double)a.s + (double)a.c;
+      tb += (double)b.s + (double)b.c;
+    }
+    red[0][tid] = ta;
+    red[1][tid] = tb;
+    __syncthreads();
+    for (int o = kT / 2; o > 0; o >>= 1) {
+      if (tid < o) {
+        red[0][tid] += red[0][tid + o];
+        red[1][tid] += red[1][tid + o];
+      }
+      __syncthreads();
+    }
+    if (tid == 0) {
+      *loss = red[0][0] * inv_count;
+      *gbout = (float)red[1][0];
+    }
+    return;
+  }
   __shared__ float red_s[8][32], red_c[8][32];
+  part += (long)blockIdx.z * nparts * cols;
   const int col = blockIdx.x * 32 + threadIdx.x;
   const int p0 = blockIdx.y * kColPer, p1 = min(nparts, p0 + kColPer);
   CSum acc;
@@ -375,42 +326,33 @@ __global__ void colsum_level1_kernel(const float* part, int nparts, int cols, fl
       o.c = red_c[k][threadIdx.x];
       t.add(o);
     }
-    mid[(long)blockIdx.y * cols + col] = t.value();
+    mid[((long)blockIdx.z * gridDim.y + blockIdx.y) * cols + col] = t.value();
   }
 }
-
-// loss = sum_p rowpart[p][0] * inv_count; gb_out = sum_p rowpart[p][1]: each thread
-// a contiguous range of parts (compensated), then a fixed tree in FP64.
-__global__ void loss_parts_kernel(const float* rowpart, int nparts, double inv_count, double* loss, float* gbout) {
-  constexpr int kT = 1024;
-  __shared__ double red[2][kT];
-  CSum a, b;
-  const int per = (nparts + kT - 1) / kT;
-  for (int p = threadIdx.x * per; p < min(nparts, (int)(threadIdx.x + 1) * per); ++p) {
-    a.add(rowpart[2 * p]);
-    b.add(rowpart[2 * p + 1]);
+// Second level: out[e] = sum_p part[p * n + e], in order of p (compensated), sixteen loads
+// ahead of their additions; blockIdx.y the array.
+struct SumArrays {
+  const float* part[16];
+  float* out[16];
+  int nparts[16];
+  long n[16];
+};
+__global__ void __launch_bounds__(128) sums_level2_kernel(const __grid_constant__ SumArrays a) {
+  const int y = blockIdx.y, nparts = a.nparts[y];
+  const long n = a.n[y], e = blockIdx.x * 128L + threadIdx.x;
+  if (e >= n) return;
+  const float* part = a.part[y] + e;
+  CSum s;
+  int p = 0;
+  for (; p + 16 <= nparts; p += 16) {
+    float v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = __ldg(part + (p + k) * n);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) s.add(v[k]);
   }
-  red[0][threadIdx.x] = (double)a.s + (double)a.c;
-  red[1][threadIdx.x] = (double)b.s + (double)b.c;
-  __syncthreads();
-  for (int o = kT / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) {
-      red[0][threadIdx.x] += red[0][threadIdx.x + o];
-      red[1][threadIdx.x] += red[1][threadIdx.x + o];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    *loss = red[0][0] * inv_count;
-    *gbout = (float)red[1][0];
-  }
-}
-
-// out[c] = sum over the parts of part[p][c] (deterministic two-level sum through mid)
-void colsum_parts(const float* part, int nparts, int cols, float* mid, float* out, cudaStream_t s) {
-  const int chunks = (nparts + kColPer - 1) / kColPer;
-  colsum_level1_kernel<<<dim3((cols + 31) / 32, chunks), dim3(32, 8), 0, s>>>(part, nparts, cols, mid);
-  sum_parts_kernel<<<nblk(cols, 256), 256, 0, s>>>(mid, chunks, cols, cols, out);
+  for (; p < nparts; ++p) s.add(part[p * n]);
+  a.out[y][e] = s.value();
 }
 
 }  // namespace
@@ -432,15 +374,13 @@ cudaError_t trainer_tc_alloc(crom_trainer* t) {
   };
   auto& c = t->tc;
   c.wh = (uint16_t*)A((size_t)(L - 1) * w * w * 2);
-  for (int h = 0; h < L; ++h) c.H.push_back((uint16_t*)A((size_t)N * w * 2));
+  for (int h = 0; h + 1 < L; ++h) c.H.push_back((uint16_t*)A((size_t)N * w * 2));  // h_{L-1} stays on the chip
   c.d0 = (uint16_t*)A((size_t)N * w * 2);
   c.d1 = (uint16_t*)A((size_t)N * w * 2);
-  c.colpart = (float*)A((size_t)tiles_m * 4 * w * 4);
-  c.colpart2 = (float*)A((size_t)tiles_m * 4 * w * 4);
+  c.colpart = (float*)A((size_t)L * tiles_m * 4 * w * 4);
   c.rowpart = (float*)A((size_t)tiles_m * 4 * 2 * 4);
-  c.resid = (float*)A((size_t)N * 4);
-  c.colmid = (float*)A((size_t)(tiles_m * 4 + kColPer - 1) / kColPer * w * 4);
-  c.split = (float*)A((size_t)kSplitsW * w * w * 4);
+  c.colmid = (float*)A((size_t)L * ((tiles_m * 4 + kColPer - 1) / kColPer) * w * 4);
+  c.split = (float*)A((size_t)(L - 1) * kSplitsW * w * w * 4);
   const int m = t->dec.m;
   c.xin = (float*)A((size_t)N * m * 4);
   c.c0 = (float*)A((size_t)t->B * w * 4);
@@ -461,6 +401,7 @@ cudaError_t trainer_decoder_tc(crom_trainer* t, double* loss_out, int num_sms, c
   const long N = (long)t->B * t->S;
   const int tiles_m = (int)((N + 127) / 128);
   const int parts = tiles_m * 4;
+  const long set = (long)parts * w, split = (long)kSplitsW * w * w;
   auto& c = t->tc;
   const TrainerLayout& lay = t->lay;
   const float* p = t->params;
@@ -481,37 +422,23 @@ cudaError_t trainer_decoder_tc(crom_trainer* t, double* loss_out, int num_sms, c
     g.B = c.wh + (size_t)(h - 1) * w * w;  // B(n, k) = W_h[n][k]
     g.ldb = w;
     g.ldo = w;
-    g.out_bf16 = c.H[h];
     g.bias = p + lay.dec_b[h];
     if (h < L - 1) {
       g.epi = kGemmEpiBiasElu;
-    } else {
+      g.out_bf16 = c.H[h];
+    } else {  // and the reverse pass of the output layer
       g.epi = kGemmEpiOut;
+      g.out_bf16 = c.d0;
+      g.colpart = c.colpart + h * set;
+      g.colpart2 = c.colpart;
+      g.rowpart = c.rowpart;
+      g.inv_count = (float)(1.0 / (double)N);
       g.wout = p + lay.dec_w[L];
       g.bout = p + lay.dec_b[L];
       g.target = t->target;
-      g.resid = c.resid;
     }
     if ((e = tc_gemm(g, num_sms, c.flag, s)) != cudaSuccess) return e;
   }
-  // delta_L, the loss terms and the output layer's column sums from h_L and the residuals
-  {
-    const unsigned blocks = (unsigned)(((long)parts + kOutWarps - 1) / kOutWarps);
-    const float inv = (float)(1.0 / (double)N);
-    if (w == 256)
-      out_delta_kernel<256><<<blocks, 32 * kOutWarps, 0, s>>>(c.H[L - 1], c.resid, p + lay.dec_w[L], N, parts, inv, c.d0,
-                                                               c.colpart, c.colpart2, c.rowpart);
-    else if (w == 128)
-      out_delta_kernel<128><<<blocks, 32 * kOutWarps, 0, s>>>(c.H[L - 1], c.resid, p + lay.dec_w[L], N, parts, inv, c.d0,
-                                                               c.colpart, c.colpart2, c.rowpart);
-    else
-      out_delta_kernel<64><<<blocks, 32 * kOutWarps, 0, s>>>(c.H[L - 1], c.resid, p + lay.dec_w[L], N, parts, inv, c.d0,
-                                                              c.colpart, c.colpart2, c.rowpart);
-  }
-  loss_parts_kernel<<<1, 1024, 0, s>>>(c.rowpart, parts, 1.0 / (double)N, loss_out ? loss_out : t->loss_dev,
-                                      gr + lay.dec_b[L]);
-  colsum_parts(c.colpart2, parts, w, c.colmid, gr + lay.dec_w[L], s);   // dL/dw_out
-  colsum_parts(c.colpart, parts, w, c.colmid, gr + lay.dec_b[L - 1], s);
   // ---- backward
   uint16_t* dcur = c.d0;
   uint16_t* dnext = c.d1;
@@ -529,12 +456,9 @@ cudaError_t trainer_decoder_tc(crom_trainer* t, double* loss_out, int num_sms, c
       g.b_mn = 1;
       g.splits = kSplitsW;
       g.epi = kGemmEpiF32;
-      g.out_f32 = c.split;
+      g.out_f32 = c.split + (h - 1) * split;
       g.ldo = w;
       if ((e = tc_gemm(g, num_sms, c.flag, s)) != cudaSuccess) return e;
-      const int sp = tc_gemm_splits_used((int)N, kSplitsW);
-      sum_parts_kernel<<<nblk((long)w * w, 256), 256, 0, s>>>(c.split, sp, (long)w * w, (long)w * w,
-                                                             gr + lay.dec_w[h]);
     }
     {  // delta[h-1] = (delta[h] W_h) s'(z_{h-1}): A(n, u) = delta[n][u], B(k, u) = W_h[u][k]
       TcGemm g;
@@ -550,12 +474,29 @@ cudaError_t trainer_decoder_tc(crom_trainer* t, double* loss_out, int num_sms, c
       g.out_bf16 = dnext;
       g.ldo = w;
       g.hprev = c.H[h - 1];
-      g.colpart = c.colpart;
+      if (h > 1) g.colpart = c.colpart + (h - 1) * set;  // db_0 below
       if ((e = tc_gemm(g, num_sms, c.flag, s)) != cudaSuccess) return e;
-      if (h > 1) colsum_parts(c.colpart, parts, w, c.colmid, gr + lay.dec_b[h - 1], s);  // db_0 below
     }
     std::swap(dcur, dnext);
   }
+  // ---- the sums: dw_out, db_1 .. db_{L-1}, the loss and db_out, dW_1 .. dW_{L-1}
+  const int mids = (parts + kColPer - 1) / kColPer;
+  sums_level1_kernel<<<dim3((w + 31) / 32, mids, L + 1), dim3(32, 8), 0, s>>>(
+      c.colpart, c.rowpart, parts, w, L, 1.0 / (double)N, c.colmid, loss_out ? loss_out : t->loss_dev, gr + lay.dec_b[L]);
+  SumArrays sums{};
+  for (int h = 0; h < L; ++h) {
+    sums.part[h] = c.colmid + (long)h * mids * w;
+    sums.out[h] = h == 0 ? gr + lay.dec_w[L] : gr + lay.dec_b[h];
+    sums.nparts[h] = mids;
+    sums.n[h] = w;
+  }
+  for (int h = 1; h < L; ++h) {
+    sums.part[L - 1 + h] = c.split + (h - 1) * split;
+    sums.out[L - 1 + h] = gr + lay.dec_w[h];
+    sums.nparts[L - 1 + h] = tc_gemm_splits_used((int)N, kSplitsW);
+    sums.n[L - 1 + h] = (long)w * w;
+  }
+  sums_level2_kernel<<<dim3(nblk((long)w * w, 128), 2 * L - 1), 128, 0, s>>>(sums);
   // ---- input layer: per-snapshot moments of delta[0], then dW_0, db_0 and dL/dq
   const int chunks = (S + kRowsB - 1) / kRowsB;
   layer0_bwd_part_kernel<<<dim3(chunks, B), w / 2, 0, s>>>(dcur, c.xin, m, S, w, c.part0);
