@@ -66,11 +66,11 @@ enum Epi { kEpiStore = 0, kEpiBiasElu = 1, kEpiTimesEluD = 2 };
 //
 // BM x BN outputs per CTA, 8 x CN per thread (two quads of rows by one or two of columns):
 // with CN = 8 shared memory delivers operands as fast as the FP32 pipe takes them (a 4 x 4
-// tile needs twice the loads).  The next 16 values of K are on their way in registers while the
-// current ones are multiplied; the row pairs feed the packed FMA.  The former 64 x 64 x 16
+// tile needs twice the loads).  The next 16 values of K (32 with four columns) are on their
+// way in registers while the current ones are multiplied; the row pairs feed the packed FMA.  The former 64 x 64 x 16
 // tiles of 4 x 4 took 81 us for 32768 x 128 x 128 (13 TFLOP/s), these 33 us (the 152 SMs
 // hold 256 tiles two to an SM, unevenly: 17 us of FMAs, then the ELU).  Weight gradients of 128
-// x 128 over 32768 rows: 196 us before, 50 us; their K ranges are fixed (the sums' order is
+// x 128 over 32768 rows: 196 us before, 35 us (50 with 16 values on their way); their K ranges are fixed (the sums' order is
 // part of the result), which leaves four warps per SM.
 struct GemmArgs {
   int M, N, K;
@@ -88,21 +88,21 @@ constexpr int kTK = 16;
 
 template <int BM, int BN, int CN, bool kAK, bool kBK>
 __global__ void __launch_bounds__(BM * BN / 8 / CN, CN == 8 ? 512 / (BM * BN / 8 / CN) : 2) gemm_kernel(GemmArgs g) {
-  constexpr int NT = BM * BN / 8 / CN, TX = BN / CN, LA = BM + 4, LB = BN + 4;
-  __shared__ __align__(16) float As[2][kTK][LA];
-  __shared__ __align__(16) float Bs[2][kTK][LB];
+  constexpr int TK = CN == 8 ? kTK : 2 * kTK, NT = BM * BN / 8 / CN, TX = BN / CN, LA = BM + 4, LB = BN + 4;
+  __shared__ __align__(16) float As[2][TK][LA];
+  __shared__ __align__(16) float Bs[2][TK][LB];
   const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
   const int i0 = blockIdx.y * BM, j0 = blockIdx.x * BN;
   const int splits = gridDim.z;
   const int kchunk = ((g.K + splits - 1) / splits + kTK - 1) / kTK * kTK;
   const int kbeg = blockIdx.z * kchunk, kend = min(g.K, kbeg + kchunk);
   // operand X (rows r < R of the tile at row0 of `rows`): float4 e of the 16 x BX tile
-  constexpr int QA = BM * kTK / 4 / NT, QB = BN * kTK / 4 / NT;
+  constexpr int QA = BM * TK / 4 / NT, QB = BN * TK / 4 / NT;
   float4 ra[QA], rb[QB];
   auto fetch = [&](const float* X, long ld, int row0, int rows, int k0, int e, bool kmajor, int BX, bool wide) -> float4 {
     float v[4];
     if (kmajor) {  // four values of k of one row
-      const int r = e / (kTK / 4), k = k0 + 4 * (e % (kTK / 4));
+      const int r = e / (TK / 4), k = k0 + 4 * (e % (TK / 4));
       const float* x = X + (long)(row0 + r) * ld + k;
       const bool in = row0 + r < rows;
       if (wide && in && k + 4 <= kend) return *reinterpret_cast<const float4*>(x);
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(BM * BN / 8 / CN, CN == 8 ? 512 / (BM * BN / 8
   };
   auto place = [&](float* S, int LD, int e, float4 v, bool kmajor, int BX) {
     if (kmajor) {
-      const int r = e / (kTK / 4), k = 4 * (e % (kTK / 4));
+      const int r = e / (TK / 4), k = 4 * (e % (TK / 4));
       S[k * LD + r] = v.x;
       S[(k + 1) * LD + r] = v.y;
       S[(k + 2) * LD + r] = v.z;
@@ -153,11 +153,11 @@ __global__ void __launch_bounds__(BM * BN / 8 / CN, CN == 8 ? 512 / (BM * BN / 8
   }
   __syncthreads();
   int buf = 0;
-  for (int k0 = kbeg; k0 < kend; k0 += kTK) {
-    const bool more = k0 + kTK < kend;
-    if (more) fetch_all(k0 + kTK);
+  for (int k0 = kbeg; k0 < kend; k0 += TK) {
+    const bool more = k0 + TK < kend;
+    if (more) fetch_all(k0 + TK);
 #pragma unroll
-    for (int kk = 0; kk < kTK; ++kk) {
+    for (int kk = 0; kk < TK; ++kk) {
       const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(&As[buf][kk][4 * ty]);
       const ulonglong2 a1 = *reinterpret_cast<const ulonglong2*>(&As[buf][kk][BM / 2 + 4 * ty]);
       const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][4 * tx]);
