@@ -38,7 +38,7 @@ namespace {
 
 constexpr int kMaxM = 3;
 constexpr int kMaxR = 32;
-constexpr int kSumGroups = 8;  // groups of partial-row chains (finish_cta)
+constexpr int kSumGroups = 16;  // groups of partial-row chains (finish_cta)
 constexpr int kKSplit = 4;  // threads per hidden unit (width <= 256 -> <= 1024 threads)
 
 enum Mode { kModeDecode = 0, kModeRecon = 1, kModeStep = 2 };
@@ -228,6 +228,15 @@ __device__ __forceinline__ double chain_sum(const double* x, int n, size_t strid
   return acc;
 }
 
+// A ticket that publishes the CTA's writes before it (ordered by a barrier) and, to
+// whoever draws the last one, those before the others (a full fence on each side of a
+// relaxed atomic cost 2 us more per launch with the groups' second ticket).
+__device__ __forceinline__ int ticket(int* counter, int n) {
+  int old;
+  asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(counter), "r"(n) : "memory");
+  return old;
+}
+
 // Output channels c of sample s at outv[s * ss + c * cs]: written out (decode,
 // reconstruction), or (step) the residuals, this CTA's partial normal equations and, in
 // the instance's last CTA, their sum and the solve.  rho [S], Amat [r][r + 1], jd [S][r]
@@ -316,8 +325,8 @@ __device__ __forceinline__ void finish_cta(const FwdParams& p, const float* outv
   const int per = max(1, 4 * p.width / ne), chains = min(per, nrows);
   const int groups = min(p.groups, chains);
   int* counters = p.counters + inst;  // CTAs, or completed groups
-  // the barrier makes every thread's rows visible to thread 0, whose fence and atomic
-  // publish them (release is cumulative)
+  // the barrier makes every thread's rows visible to thread 0, whose ticket publishes them
+  // (release is cumulative)
   __syncthreads();
   if (groups > 1) {
     int* gcount = p.group_counters + (size_t)inst * p.groups;
@@ -328,10 +337,8 @@ __device__ __forceinline__ void finish_cta(const FwdParams& p, const float* outv
         for (int t = row0; t < row0 + rows; ++t) mine += t % per % groups == tid;
         for (int j = tid; j < chains; j += groups) all += (nrows - j + per - 1) / per;
       }
-      __threadfence();
-      const bool last = mine > 0 && atomicAdd(&gcount[tid], mine) == all - mine;
+      const bool last = mine > 0 && ticket(&gcount[tid], mine) == all - mine;
       const unsigned d = __ballot_sync(0xffffffffu, last);
-      __threadfence();
       if (tid == 0) s_groups = d;
     }
     __syncthreads();
@@ -350,14 +357,10 @@ __device__ __forceinline__ void finish_cta(const FwdParams& p, const float* outv
     __syncthreads();
     if (tid == 0) {
       const int n = __popc(done);
-      __threadfence();
-      s_flag = atomicAdd(counters, n) == groups - n;
-      __threadfence();
+      s_flag = ticket(counters, n) == groups - n;
     }
   } else if (tid == 0) {
-    __threadfence();
-    s_flag = atomicAdd(counters, 1) == ntiles - 1;
-    __threadfence();
+    s_flag = ticket(counters, 1) == ntiles - 1;
   }
   __syncthreads();
   if (!s_flag) return;
@@ -609,10 +612,23 @@ cudaError_t launch_fwd(FwdParams& p, FwdKernel kind, dim3 grid, cudaStream_t s) 
   if (kind != kFwdGeneral) {
     // more threads than the products need fetch the weights and share the activation passes
     const size_t smem = small_smem_bytes(W, p.S, p.C, p.m, p.r, p.hidden);
-    auto small = [&](auto k64, auto k128, auto any) {
-      return W == 64 ? go(k64, kSmallThreads, smem) : W == 128 ? go(k128, kSmallThreads, smem) : go(any, kSmallThreads, smem);
-    };
-    return small(fwd_small_kernel<64>, fwd_small_kernel<128>, fwd_small_kernel<0>);
+    const auto kernel = W == 64 ? fwd_small_kernel<64> : W == 128 ? fwd_small_kernel<128> : fwd_small_kernel<0>;
+    if (p.mode != kModeStep) return go(kernel, kSmallThreads, smem);
+    // a chain of launches that each wait for one CTA's solve: the next one's CTAs start and
+    // load the decoder meanwhile (200 samples, width 128: 72 us a step of two without, 69 with)
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kSmallThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, p);
   }
   const size_t smem = fwd_smem_bytes(W, p.S, p.C, p.m, p.r, &p.LD);
   return p.jvp_seed ? go(fwd_fp32_jvp_kernel, W * kKSplit, smem) : go(fwd_fp32_kernel, W * kKSplit, smem);

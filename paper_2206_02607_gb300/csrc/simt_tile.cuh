@@ -16,7 +16,7 @@
 //  * fwd_small_kernel: latency, for problems of too few samples to fill the GPU that
 //    way (one instance of a few hundred samples).  One or two samples per CTA, the
 //    quarters of K go to different threads, a whole layer of weights is in flight while
-//    the one before is used.  A step of 200 samples, width 128: 150 -> 72 us, of which
+//    the one before is used.  A step of 200 samples, width 128: 150 -> 67 us, of which
 //    one CTA's reduction and solve take a third.
 #pragma once
 
@@ -94,7 +94,7 @@ struct TileShared {
   int* code;    // [S]
 };
 __device__ __forceinline__ bool stage_inputs(const FwdParams& p, const TileShared& t, const double* w1q,
-                                             const float* b1, int inst, int first, int ns) {
+                                             const float* b1, int inst, int first, int ns, bool have_q = false) {
   const int tid = threadIdx.x, NT = blockDim.x, S = p.S, m = p.m, r = p.r, W = p.width;
   for (int i = tid; i < S * m; i += NT) {
     const int s = i / m, k = i % m;
@@ -107,11 +107,11 @@ __device__ __forceinline__ bool stage_inputs(const FwdParams& p, const TileShare
     one = t.code[0] == t.code[ns - 1];
     const int n = one ? r : S * r;
     for (int i = tid; i < n; i += NT) t.qs[i] = p.q[(size_t)t.code[i / r] * r + i % r];
-  } else {
+  } else if (!have_q) {
     const double* q = p.mode == kModeStep ? p.qio + (size_t)inst * r : p.q + (size_t)blockIdx.y * r;
     for (int j = tid; j < r; j += NT) t.qs[j] = q[j];
   }
-  if (p.diff)
+  if (p.diff && !have_q)
     for (int j = tid; j < r; j += NT) t.dqs[j] = p.qio[(size_t)inst * r + j] - p.qbase[(size_t)inst * r + j];
   __syncthreads();
   // FP64 is a slow pipe on this GPU (2 FMA per clock and SM): one thread per unit, not
@@ -527,7 +527,7 @@ __host__ __device__ constexpr int small_rows(int W) { return W <= 128 ? W / 4 : 
 constexpr int kSmallThreads = 512;
 
 // Everything the CTA will need from global memory is requested up front (first layer,
-// biases, output row, the first weight stage), so that one memory latency is paid, not
+// biases, output row, the first two weight stages), so that one memory latency is paid, not
 // one per layer.  kW: the width, 0 = any (p.width).
 template <int kW>
 __global__ void __launch_bounds__(kSmallThreads, 1) fwd_small_kernel(FwdParams p) {
@@ -557,9 +557,6 @@ __global__ void __launch_bounds__(kSmallThreads, 1) fwd_small_kernel(FwdParams p
   ts.zdf = ts.csf + W;
   ts.code = reinterpret_cast<int*>(ts.zdf + W);
 
-  int inst, first, ns, ntiles, total;
-  if (!tile_range(p, inst, first, ns, ntiles, total)) return;
-
   auto copy = [&](float* dst, const float* src, int n) {
     for (int i = tid * 4; i < n; i += NT * 4) cp_async16(dst + i, src + i);
   };
@@ -585,11 +582,29 @@ __global__ void __launch_bounds__(kSmallThreads, 1) fwd_small_kernel(FwdParams p
   };
   if (stages > 0) fetch(0, 0, NT);
   cp_async_commit();
+  if (stages > 1) fetch(1, 0, NT);
+  cp_async_commit();
+  // A step's launches overlap: up to here a CTA reads the decoder alone, while the last
+  // CTA of the launch before may still add and solve (a third of its time, on one SM).
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const bool step = p.mode == kModeStep && tid < r;  // its codes come along with its range
+  const double qk = step ? p.qio[(size_t)blockIdx.x * r + tid] : 0.0;
+  const double qn = step && p.diff ? p.qbase[(size_t)blockIdx.x * r + tid] : 0.0;
+  int inst, first, ns, ntiles, total;
+  if (!tile_range(p, inst, first, ns, ntiles, total)) {
+    cp_async_wait<0>();
+    return;
+  }
+  if (step) {
+    ts.qs[tid] = qk;
+    ts.dqs[tid] = qk - qn;
+  }
   if (NP < NPP)
     for (int u = tid; u < W; u += NT)
       for (int c = NP; c < NPP; ++c) H[u * LD + c] = 0.f;  // padding columns
-  cp_async_wait<1>();  // the first-layer group; stage_inputs has a barrier before its first use
-  const bool one = stage_inputs(p, ts, wqs, b1s, inst, first, ns);
+  cp_async_wait<2>();  // the first-layer group; stage_inputs has a barrier before its first use
+  const bool one = stage_inputs(p, ts, wqs, b1s, inst, first, ns, p.mode == kModeStep);
   const int ox = 1 + p.diff, n2 = (p.second == kSecondPerK) ? m : (p.second == kSecondLap ? 1 : 0);
   const int o2 = ox + p.nx, oq = o2 + n2;
   // activation items (unit, sample, part): part 0 the special channels, the others a
@@ -657,9 +672,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) fwd_small_kernel(FwdParams p
         for (int e = 0; e < 4; ++e) acc[t][a][e] = 0ull;
     for (int st = 0; st < per_layer; ++st) {
       const int g = l * per_layer + st;
-      cp_async_wait<0>();
+      if (g == 0) cp_async_wait<1>();
+      else cp_async_wait<0>();
       __syncthreads();
-      if (g + 1 < stages) fetch(g + 1, f0, fn);
+      if (g > 0 && g + 1 < stages) fetch(g + 1, f0, fn);
       cp_async_commit();
       if (active) {
         const float* w = Ws + (g & 1) * stage_floats + ks * qfloats + u0;
