@@ -39,7 +39,7 @@ using namespace tc;
 constexpr int kBM = 128, kBK = 64, kStages = 3;
 // Column parts of a tile's epilogue, a warp of each for every 32 rows.  Two hold the issue
 // slots at 40 %, waiting on tensor memory, shuffles and the staging rows; four hide that
-// (the s' epilogue 88 -> 80 us at 2^18 rows of 256, bias + ELU 52 -> 50 us) where the parts
+// (the s' epilogue 88 -> 75 us at 2^18 rows of 256, bias + ELU 52 -> 50 us) where the parts
 // keep 32 columns.  The output layer's sum over the columns is one chain per half.
 template <int kBN, int kEpi>
 constexpr int kParts = kBN >= 128 && (kEpi == kGemmEpiTimesEluD || kEpi == kGemmEpiBiasElu) ? 4 : 2;
@@ -166,17 +166,13 @@ struct Staging {
 #pragma unroll
     for (int j = 0; j < 4; ++j) d[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
   }
-  __device__ __forceinline__ void get32(int lane, int c0, float (&v)[32]) const {
-    const uint4* sp = reinterpret_cast<const uint4*>(base + lane * kSt + c0);
+  __device__ __forceinline__ void get8(int lane, int c0, float (&v)[8]) const {
+    const uint4 q = *reinterpret_cast<const uint4*>(base + lane * kSt + c0);
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint4 q = sp[j];
-      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        v[8 * j + 2 * i] = __uint_as_float(w[i] << 16);
-        v[8 * j + 2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-      }
+    for (int i = 0; i < 4; ++i) {
+      v[2 * i] = __uint_as_float(w[i] << 16);
+      v[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
     }
   }
   // columns col0 .. col0 + kW - 1 of rows row0 .. row0 + 31 (those < M) of the [M][ld]
@@ -411,6 +407,11 @@ __global__ void __launch_bounds__(64 + 128 * kParts<kBN, kEpi>, 1)
       // h_{l-1} of the tile's rows does not depend on the accumulator: the first tile
       // reads it here, later ones were fetched during the previous tile's stores
       if (kEpi == kGemmEpiTimesEluD && local == 0) stg.load_rows(g.hprev, g.ldo, row0, cb, g.M, lane);
+      // the next tile's rows of h_{l-1} are on their way while this one is worked on
+      const int tn = t + gridDim.x;
+      uint4 R[Staging<kCols>::kFetch];
+      if (kEpi == kGemmEpiTimesEluD && tn < tiles)
+        stg.fetch_rows(g.hprev, g.ldo, (tn % g.tiles_m) * kBM + q * 32, cb, g.M, lane, R);
       g_wait(bars, &bars->tfull[acc], tphase[acc]);
       tphase[acc] ^= 1;
       tc_fence_after();
@@ -445,10 +446,13 @@ __global__ void __launch_bounds__(64 + 128 * kParts<kBN, kEpi>, 1)
           for (int j = 0; j < 32; ++j) v[j] = elu_g(v[j] + sbias[c0 + j]);
           stg.put32(lane, c0, v);
         } else if (kEpi == kGemmEpiTimesEluD) {
-          float hp[32];
-          stg.get32(lane, c0, hp);
 #pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = in ? v[j] * elud_from_h(hp[j]) : 0.f;
+          for (int j = 0; j < 32; j += 8) {
+            float hp[8];
+            stg.get8(lane, c0 + j, hp);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[j + i] = in ? v[j + i] * elud_from_h(hp[i]) : 0.f;
+          }
           stg.put32(lane, c0, v);                    // in place of the h values just read
           if (g.colpart) {  // column sums of delta over this warp's rows
             const float cs = warp_colsum32(v, lane);
@@ -463,10 +467,6 @@ __global__ void __launch_bounds__(64 + 128 * kParts<kBN, kEpi>, 1)
       if (lane == 0) mbar_arrive(&bars->tempty[acc]);
       if (kEpi == kGemmEpiBiasElu) stg.store_rows(g.out_bf16, g.ldo, row0, cb, g.M, lane);
       if (kEpi == kGemmEpiTimesEluD) {
-        // the next tile's h_{l-1} rows are loaded while this tile's delta rows are stored
-        const int tn = t + gridDim.x;
-        uint4 R[Staging<kCols>::kFetch];
-        if (tn < tiles) stg.fetch_rows(g.hprev, g.ldo, (tn % g.tiles_m) * kBM + q * 32, cb, g.M, lane, R);
         stg.store_rows(g.out_bf16, g.ldo, row0, cb, g.M, lane);
         if (tn < tiles) stg.put_rows(lane, R);
       }
