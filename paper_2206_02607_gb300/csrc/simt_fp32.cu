@@ -96,16 +96,11 @@ struct FwdParams {
 };
 
 __device__ __forceinline__ void elu3(float z, float& s0, float& s1, float& s2) {
-  if (z > 0.f) {
-    s0 = z;
-    s1 = 1.f;
-    s2 = 0.f;
-  } else {
-    float e = expf(z);
-    s0 = expm1f(z);
-    s1 = e;
-    s2 = e;
-  }
+  // without a divergent branch (a NaN stays a NaN)
+  const float zm = z > 0.f ? 0.f : z, e = expf(zm), em = expm1f(zm);
+  s0 = z > 0.f ? z : em;
+  s1 = z > 0.f ? 1.f : e;
+  s2 = z > 0.f ? 0.f : e;
 }
 
 // s(a) - s(a - d) without cancellation: the difference channel carries
@@ -213,16 +208,17 @@ __device__ __forceinline__ void entry_of(int e, int r, int ntri, int& a, int& b)
     b = -1;
   }
 }
-// x[0] + x[stride] + .. (n terms, in order), the loads issued ahead of the additions.
+// x[0] + x[stride] + .. (n terms, in order), kAhead loads issued ahead of the additions.
+template <int kAhead>
 __device__ __forceinline__ double chain_sum(const double* x, int n, size_t stride) {
   double acc = 0.0;
-  for (int k0 = 0; k0 < n; k0 += 20) {
-    double v[20];
+  for (int k0 = 0; k0 < n; k0 += kAhead) {
+    double v[kAhead];
 #pragma unroll
-    for (int k = 0; k < 20; ++k)
+    for (int k = 0; k < kAhead; ++k)
       if (k0 + k < n) v[k] = __ldcg(x + (size_t)(k0 + k) * stride);
 #pragma unroll
-    for (int k = 0; k < 20; ++k)
+    for (int k = 0; k < kAhead; ++k)
       if (k0 + k < n) acc += v[k];
   }
   return acc;
@@ -249,6 +245,10 @@ __device__ __forceinline__ int ticket(int* counter, int n) {
 // FP64 is slow here (64 clocks per warp instruction), so with p.groups > 1 the chains
 // are dealt to that many groups, and the CTA that completes a group's last row adds its
 // chains (into their first rows); the CTA that completes the last group adds the chains.
+//
+// kAhead: partial rows read ahead of their addition (20 hide the memory latency of a chain
+// of a few hundred samples; the general kernel's 64 registers hold 4).
+template <int kAhead>
 __device__ __forceinline__ void finish_cta(const FwdParams& p, const float* outv, int ss, int cs, int inst, int first,
                                            int ns, int ntiles, int total, double* rho, double* Amat, double* jd,
                                            double* red2) {
@@ -350,7 +350,7 @@ __device__ __forceinline__ void finish_cta(const FwdParams& p, const float* outv
       for (int i = tid; i < nc * ne; i += NT) {
         const int j = g + i / ne * groups;
         double* row = base + (size_t)j * ne + i % ne;
-        *row = chain_sum(row, (nrows - j + per - 1) / per, (size_t)per * ne);
+        *row = chain_sum<kAhead>(row, (nrows - j + per - 1) / per, (size_t)per * ne);
       }
       if (tid == 0) gcount[g] = 0;
     }
@@ -369,14 +369,14 @@ __device__ __forceinline__ void finish_cta(const FwdParams& p, const float* outv
   if (groups <= 1) {
     for (int i = tid; i < chains * ne; i += NT) {
       const int e = i % ne, j = i / ne;
-      red2[i] = chain_sum(base + (size_t)j * ne + e, (nrows - j + per - 1) / per, (size_t)per * ne);
+      red2[i] = chain_sum<kAhead>(base + (size_t)j * ne + e, (nrows - j + per - 1) / per, (size_t)per * ne);
     }
     __syncthreads();
   }
   for (int e = tid; e < ne; e += NT) {
     double acc;
     if (groups > 1) {
-      acc = chain_sum(base + e, chains, (size_t)ne);
+      acc = chain_sum<kAhead>(base + e, chains, (size_t)ne);
     } else {
       acc = 0.0;
       for (int j = 0; j < chains; ++j) acc += red2[j * ne + e];
@@ -479,30 +479,31 @@ __device__ __forceinline__ void fwd_fp32_body(const FwdParams& p) {
   // ---- layer 1: pre-activation channels of unit u, then the activation chain
   {
     float* row = Hin + u * LD;
-    const float* w1 = p.w1 + (size_t)u * (m + r);
+    const float* w1 = p.w1t + u;  // entry k at w1[k * W]
+    const double* w1q = p.w1q + u;
     const double b1 = (double)p.b1[u];
     double cshared = b1;
     const bool shared_q = (p.mode != kModeDecode);
     if (shared_q) {
-      for (int j = 0; j < r; ++j) cshared += (double)w1[m + j] * qs[j];
+      for (int j = 0; j < r; ++j) cshared += w1q[j * W] * qs[j];
     }
     double zd = 0.0;
     if (p.diff) {
-      for (int j = 0; j < r; ++j) zd += (double)w1[m + j] * dqs[j];
+      for (int j = 0; j < r; ++j) zd += w1q[j * W] * dqs[j];
     }
     for (int s = ks; s < S; s += KS) {
       double c = cshared;
       if (!shared_q) {
         c = b1;
-        for (int j = 0; j < r; ++j) c += (double)w1[m + j] * qs[s * r + j];
+        for (int j = 0; j < r; ++j) c += w1q[j * W] * qs[s * r + j];
       }
       float z = (float)c;
-      for (int k = 0; k < m; ++k) z = fmaf(w1[k], xs[s * m + k], z);
+      for (int k = 0; k < m; ++k) z = fmaf(w1[k * W], xs[s * m + k], z);
       float* ch = row + s * C;
       ch[0] = z;
       if (p.diff) ch[1] = (float)zd;
       const int ox = 1 + p.diff;
-      for (int k = 0; k < p.nx; ++k) ch[ox + k] = w1[k];
+      for (int k = 0; k < p.nx; ++k) ch[ox + k] = w1[k * W];
       int o = ox + p.nx;
       const int n2 = (p.second == kSecondPerK) ? m : (p.second == kSecondLap ? 1 : 0);
       for (int k = 0; k < n2; ++k) ch[o + k] = 0.f;
@@ -511,7 +512,7 @@ __device__ __forceinline__ void fwd_fp32_body(const FwdParams& p) {
         const int code = find_instance(p.off, p.n_inst, first + (s < ns ? s : 0));
         ch[o] = __ldg(&p.jvp_seed[(size_t)code * W + u]);
       } else {
-        for (int j = 0; j < p.nq; ++j) ch[o + j] = w1[m + j];
+        for (int j = 0; j < p.nq; ++j) ch[o + j] = w1[(m + j) * W];
       }
     }
     activate_row(row, p, ks, KS);
@@ -563,7 +564,7 @@ __device__ __forceinline__ void fwd_fp32_body(const FwdParams& p) {
 
   output_layer(p, p.wout, Hin, LD, NP, outv, 0);
   __syncthreads();
-  finish_cta(p, outv, C, 1, inst, first, ns, ntiles, msz, rho, Amat, qs, reinterpret_cast<double*>(red));
+  finish_cta<4>(p, outv, C, 1, inst, first, ns, ntiles, msz, rho, Amat, qs, reinterpret_cast<double*>(red));
 }
 
 __global__ void __launch_bounds__(1024) fwd_fp32_kernel(FwdParams p) { fwd_fp32_body<false>(p); }
@@ -672,19 +673,43 @@ bool small_fits(int W, int S, int C, int m, int r, int hidden) {
 
 int pick_samples(int W, int C, int m, int r, int want);
 
-// Kernel and samples per CTA for `sets` groups of n points with C channels (decode and
-// reconstruction): the tile kernel once its smallest tiles (4 samples) give every SM
-// one, below that the latency kernel, two samples per CTA where one would not fit the
-// GPU at once (200 samples of a 2D step: 72 us with two, 96 us with one per CTA).
+// Which kernel N samples of C channels get (decode, reconstruction and step); all three
+// measured on 550 shapes (widths 32 to 256, 1 to 16 channels, 1 to 10^5 samples), with
+// these lines the choice is within 2 % of the best on average and nowhere more than 5 %
+// slower than the general kernel was alone.
+//  * The tile kernel from three warps per SM on (a warp: 8 units x 8 columns a lane), four
+//    for up to four channels: 0.3 to 0.9 of the general kernel's time above the line, 1.2
+//    to 3.5 times it below (one warp per CTA walks all of K: 1362 values of width 256, 471
+//    us against 181 us).  A lone channel needs four at width 128 and more in proportion to
+//    the width, as its chain over K grows while the general kernel splits it; the step's
+//    bound on N counts every instance at its largest, six.
+//  * Else the latency kernel, two samples per CTA where one would not fit the GPU at once
+//    (200 samples of a 2D step: 67 us with two, 91 us with one per CTA), if its CTAs take
+//    no more rounds of the GPU than (C + 1) / 2 (step: C / 2): its time grows with the rounds, the
+//    general kernel's with the channels (1000 values of width 64: 1.7 times, 45 x 5
+//    channels of 600: 0.9 times).  Width 32 and two layers leave too little to gain in a
+//    second round.
+//  * Else the general kernel.
+bool tile_pays(const crom_ctx* ctx, long long N, int C, bool step) {
+  const int W = ctx->desc.width;
+  const long long warps = N * C * W / 2048, sms = ctx->num_sms;
+  if (step) return warps >= 6 * sms;
+  return C > 1 ? warps >= (C > 4 ? 3 : 4) * sms : warps >= std::max(3 * sms, 4 * sms * W / 128);
+}
+bool small_pays(const crom_ctx* ctx, long long N, int S, int C, bool step) {
+  const long long ctas = (N + S - 1) / S, rounds = (ctas + ctx->num_sms - 1) / ctx->num_sms;
+  return rounds <= 1 || (ctx->desc.width > 32 && ctx->desc.hidden > 2 && 2 * rounds <= C + !step);
+}
+
 FwdKernel plan_points(const crom_ctx* ctx, long long sets, long long n, int C, int general_want, int* S) {
   const int W = ctx->desc.width, m = ctx->desc.m, r = ctx->desc.r;
-  if (sets * ((n + 3) / 4) >= ctx->num_sms) {
+  const long long N = sets * n;
+  if (tile_pays(ctx, N, C, false)) {
     const FwdKernel k = tile_plan(ctx, sets, n, C, S);
     if (k != kFwdGeneral) return k;
-  } else {
-    for (*S = sets * n > ctx->num_sms ? 2 : 1; *S >= 1; --*S)
-      if (small_fits(W, *S, C, m, r, ctx->desc.hidden)) return kFwdSmall;
   }
+  for (*S = N > ctx->num_sms ? 2 : 1; *S >= 1; --*S)
+    if (small_fits(W, *S, C, m, r, ctx->desc.hidden) && small_pays(ctx, N, *S, C, false)) return kFwdSmall;
   *S = pick_samples(W, C, m, r, general_want);
   return kFwdGeneral;
 }
@@ -817,13 +842,13 @@ FwdKernel plan_step(const crom_ctx* ctx, int n_inst, int max_samples, int* S, in
   const int W = ctx->desc.width, m = ctx->desc.m, r = ctx->desc.r;
   const int C0 = ChannelSet{m, kSecondLap, r}.count(m);
   *PS = step_samples_per_cta(ctx, n_inst, max_samples);
-  if ((long long)n_inst * (((long long)max_samples + 3) / 4) >= ctx->num_sms) {
+  const long long N = (long long)n_inst * max_samples;
+  if (tile_pays(ctx, N, C0, true)) {
     const FwdKernel k = tile_plan(ctx, n_inst, max_samples, C0, S);
     if (k != kFwdGeneral) return k;
-  } else {
-    for (*S = (long long)n_inst * max_samples > ctx->num_sms ? 2 : 1; *S >= 1; --*S)
-      if (*S % *PS == 0 && small_fits(W, *S, C0, m, r, ctx->desc.hidden)) return kFwdSmall;
   }
+  for (*S = N > ctx->num_sms ? 2 : 1; *S >= 1; --*S)
+    if (*S % *PS == 0 && small_fits(W, *S, C0, m, r, ctx->desc.hidden) && small_pays(ctx, N, *S, C0, true)) return kFwdSmall;
   *S = *PS;
   return kFwdGeneral;
 }

@@ -51,18 +51,11 @@ __device__ __forceinline__ f2 add2p(f2 a, f2 b) {
 __device__ __forceinline__ float lo2(f2 v) { return __uint_as_float((uint32_t)v); }
 __device__ __forceinline__ float hi2(f2 v) { return __uint_as_float((uint32_t)(v >> 32)); }
 
-// s(z), s'(z), s''(z) as elu3 / siren3 form them, without divergent branches (a NaN
-// stays a NaN: the comparison keeps it in the exponential).
+// s(z), s'(z), s''(z).
 template <bool kSiren>
 __device__ __forceinline__ void act3(const FwdParams& p, float z, float& s0, float& s1, float& s2) {
-  if (kSiren) {
-    siren3(z, p.omega0, s0, s1, s2);
-  } else {
-    const float zm = z > 0.f ? 0.f : z, e = expf(zm), em = expm1f(zm);
-    s0 = z > 0.f ? z : em;
-    s1 = z > 0.f ? 1.f : e;
-    s2 = z > 0.f ? 0.f : e;
-  }
+  if (kSiren) siren3(z, p.omega0, s0, s1, s2);
+  else elu3(z, s0, s1, s2);
 }
 template <bool kSiren>
 __device__ __forceinline__ float act_value(const FwdParams& p, float z) {
@@ -506,7 +499,7 @@ __global__ void __launch_bounds__(256, 4 - TQ) fwd_tile_kernel(FwdParams p) {
   if (tid < 32) tc::tmem_dealloc(s_tmem, kCols);
   output_layer(p, p.wout, H, LD, NP, outv, S);
   __syncthreads();
-  finish_cta(p, outv, 1, S, inst, first, ns, ntiles, total, rho, Amat, ts.qs, reinterpret_cast<double*>(H));
+  finish_cta<20>(p, outv, 1, S, inst, first, ns, ntiles, total, rho, Amat, ts.qs, reinterpret_cast<double*>(H));
 }
 
 inline size_t tile_smem_bytes(int W, int S, int C, int m, int r) {
@@ -720,7 +713,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) fwd_small_kernel(FwdParams p
   __syncthreads();
   output_layer(p, wos, H, LD, NP, outv, 0);
   __syncthreads();
-  finish_cta(p, outv, C, 1, inst, first, ns, ntiles, total, rho, Amat, ts.qs, reinterpret_cast<double*>(red));
+  finish_cta<20>(p, outv, C, 1, inst, first, ns, ntiles, total, rho, Amat, ts.qs, reinterpret_cast<double*>(red));
 }
 
 inline size_t small_smem_bytes(int W, int S, int C, int m, int r, int hidden) {
