@@ -764,7 +764,7 @@ def main():
     train_ms = time_train(crom.CROM_PREC_BF16_MIXED, 10)
     pts = Bt * St
     train_flops = pts * 6 * (2 * (2 + rt) * wt + 2 * (Lt - 1) * wt * wt + 2 * wt) / 2
-    train_bytes = (7 * Lt - 3) * pts * wt * 2
+    train_bytes = (7 * Lt - 5) * pts * wt * 2
     tr.close()
 
     next_rows = measure_next_rows(crom, gen, ctx, w, q0, alpha, s_off, samples, status, stream, flush, local)
@@ -825,17 +825,20 @@ def main():
                               "note": "crom_rollout: 1000 steps replayed from a cached CUDA graph, no L2 flush"},
             "fom_advdiff2d": {"node_steps_per_s": fom_nodes / (fom_ms * 1e-3), "ms_per_step": fom_ms,
                               "gbs_algorithmic": fom_gbs, "frac_of_measured_hbm": fom_gbs / hbm,
-                              "workload": "512 periodic 256^2 fields, 16 B per node-step (u, ax, ay read, u written)"},
+                              "bytes_note": "16 B per node-step (u, ax, ay read, u written), what a launch per step "
+                                            "moves; the steps of a call stay on the chip, so this exceeds HBM",
+                              "workload": "512 periodic 256^2 fields, several steps per call"},
             "next_rows": next_rows,
             "fom_heat2d": {"node_steps_per_s": heat_nodes / (heat_ms * 1e-3), "ms_per_step": heat_ms,
                            "gbs_algorithmic": heat_gbs, "frac_of_measured_hbm": heat_gbs / hbm,
-                           "workload": "1024 zero-flux 256^2 fields, 8 B per node-step (u read and written)"},
+                           "bytes_note": "8 B per node-step (u read and written), as above",
+                           "workload": "1024 zero-flux 256^2 fields, several steps per call"},
             "training": {"point_samples_per_s": pts / (train_ms * 1e-3), "ms_per_step": train_ms,
                          "tflops_algorithmic": train_flops / (train_ms * 1e-3) / 1e12,
                          "frac_of_measured_bf16": train_flops / (train_ms * 1e-3) / 1e12 / peak_tf,
                          "hbm_gbs_algorithmic": train_bytes / (train_ms * 1e-3) / 1e9,
                          "frac_of_measured_hbm": train_bytes / (train_ms * 1e-3) / 1e9 / hbm,
-                         "bytes_note": "decoder pass: 7 L - 3 reads or writes of a [B*S][w] bf16 array "
+                         "bytes_note": "decoder pass: 7 L - 5 reads or writes of a [B*S][w] bf16 array "
                                        "per step (activations, deltas), the roofline that binds here",
                          "precision": "library tcgen05 GEMMs with fused epilogues, bf16 operands, FP32 "
                                       "accumulation and master weights",
