@@ -136,12 +136,13 @@ __global__ void layer0_bwd_part_kernel(const uint16_t* delta, const float* x_in,
   const uint32_t* dp = reinterpret_cast<const uint32_t*>(delta + r0 * w + u);
   const int ldw = w / 2;
   int i = 0;
-  for (; i + 4 <= nr; i += 4) {
-    uint32_t d4[4];
+  constexpr int kAhead = 16;  // rows read before they are added (four: 33 us for 2^18 rows of 256, sixteen: 29)
+  for (; i + kAhead <= nr; i += kAhead) {
+    uint32_t d4[kAhead];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) d4[k] = __ldg(dp + (long)(i + k) * ldw);
+    for (int k = 0; k < kAhead; ++k) d4[k] = __ldg(dp + (long)(i + k) * ldw);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < kAhead; ++k) {
       const float da = bf16_val((uint16_t)(d4[k] & 0xffffu)), db = bf16_val((uint16_t)(d4[k] >> 16));
       sa += da;
       sb += db;
