@@ -682,23 +682,25 @@ int pick_samples(int W, int C, int m, int r, int want);
 //    to 3.5 times it below (one warp per CTA walks all of K: 1362 values of width 256, 471
 //    us against 181 us).  A lone channel needs four at width 128 and more in proportion to
 //    the width, as its chain over K grows while the general kernel splits it; the step's
-//    bound on N counts every instance at its largest, six.
+//    bound on N counts every instance at its largest, six, in 1D (few
+//    channels, short uneven instances) ten.
 //  * Else the latency kernel, two samples per CTA where one would not fit the GPU at once
 //    (200 samples of a 2D step: 67 us with two, 91 us with one per CTA), if its CTAs take
 //    no more rounds of the GPU than (C + 1) / 2 (step: C / 2): its time grows with the rounds, the
 //    general kernel's with the channels (1000 values of width 64: 1.7 times, 45 x 5
 //    channels of 600: 0.9 times).  Width 32 and two layers leave too little to gain in a
-//    second round.
+//    second round, three layers in a third.
 //  * Else the general kernel.
 bool tile_pays(const crom_ctx* ctx, long long N, int C, bool step) {
   const int W = ctx->desc.width;
   const long long warps = N * C * W / 2048, sms = ctx->num_sms;
-  if (step) return warps >= 6 * sms;
+  if (step) return warps >= (ctx->desc.m == 1 ? 10 : 6) * sms;
   return C > 1 ? warps >= (C > 4 ? 3 : 4) * sms : warps >= std::max(3 * sms, 4 * sms * W / 128);
 }
 bool small_pays(const crom_ctx* ctx, long long N, int S, int C, bool step) {
   const long long ctas = (N + S - 1) / S, rounds = (ctas + ctx->num_sms - 1) / ctx->num_sms;
-  return rounds <= 1 || (ctx->desc.width > 32 && ctx->desc.hidden > 2 && 2 * rounds <= C + !step);
+  const int hidden = ctx->desc.hidden;
+  return rounds <= 1 || (ctx->desc.width > 32 && hidden > 2 && (hidden > 3 || rounds <= 2) && 2 * rounds <= C + !step);
 }
 
 FwdKernel plan_points(const crom_ctx* ctx, long long sets, long long n, int C, int general_want, int* S) {
