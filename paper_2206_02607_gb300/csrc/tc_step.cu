@@ -821,16 +821,14 @@ __device__ __forceinline__ bool decode_chunk(Lane& c, const StepParams& p, int a
 }
 
 // ---------------- split mode
-// Tiles of instance i at this iteration; 0 where it takes no part (an invalid range, or a
-// status other than OK after an earlier iteration).
-template <int kSS, Mode kMode>
-__device__ __forceinline__ int iter_tiles(const StepParams& p, int i) {
+// Tiles of instance i; 0 where its range is invalid.  From the offsets alone, in every
+// iteration: the CTAs of a launch must all lay out the same tiles, and a launch writes
+// the statuses of the instances it completes while a CTA that waited for an SM (another
+// stream's kernel held it) has yet to start.
+template <int kSS>
+__device__ __forceinline__ int deal_tiles(const StepParams& p, int i) {
   const int o0 = p.off[i], M = p.off[i + 1] - o0;
-  if (kMode == kIterLater) {
-    if (p.status[i] != CROM_OK) return 0;
-  } else if (M < p.r || M > p.max_samples || o0 < 0 || o0 + M > p.n_samples) {
-    return 0;
-  }
+  if (M < p.r || M > p.max_samples || o0 < 0 || o0 + M > p.n_samples) return 0;
   return (M + kSS - 1) / kSS;
 }
 
@@ -839,7 +837,11 @@ __device__ __forceinline__ int iter_tiles(const StepParams& p, int i) {
 // of p.rows, and the group that completes an instance's last tile adds the rows in order
 // of the tiles (the order in which a group that owns the whole instance adds them: the
 // same bits) and solves.  No group waits for another.  A bounded wait that runs out marks
-// the instances of the group's range, which then end as TIMEOUT.
+// the instances of the group's range, which then end as TIMEOUT.  An instance that failed
+// in an earlier iteration keeps its place in the row, but nothing is done for it: every
+// group that comes to it skips it, since its status no longer changes, and the status of
+// one that has not failed changes only after all its tiles are counted, this group's
+// among them.
 template <int kM, bool kLoP, Mode kMode>
 __device__ __forceinline__ bool run_iteration(Lane& c, const StepParams& p, Own& own, uint8_t* scratch, int* part, bool ok) {
   constexpr int kSS = 2 * tile_s0<kLoP>();
@@ -851,7 +853,7 @@ __device__ __forceinline__ bool run_iteration(Lane& c, const StepParams& p, Own&
   const int per = (p.n_inst + kThreads - 1) / kThreads, i0 = min(p.n_inst, tid * per), i1 = min(p.n_inst, i0 + per);
   int sum = 0;
   for (int i = i0; i < i1; ++i) {
-    const int nt = iter_tiles<kSS, kMode>(p, i);
+    const int nt = deal_tiles<kSS>(p, i);
     if (kMode == kIterFirst && nt == 0 && blockIdx.x == 0) p.status[i] = CROM_ERR_INVALID_ARG;
     prefix[i] = sum;
     sum += nt;
@@ -887,9 +889,14 @@ __device__ __forceinline__ bool run_iteration(Lane& c, const StepParams& p, Own&
   }
   __syncthreads();  // the operand blocks are free again
   for (; a < b; ++inst) {
-    const int nt = iter_tiles<kSS, kMode>(p, inst);
+    const int nt = deal_tiles<kSS>(p, inst);
     if (nt == 0) continue;
     const int e = min(b, base + nt), o0 = p.off[inst], M = p.off[inst + 1] - o0;
+    if (kMode == kIterLater && p.status[inst] != CROM_OK) {
+      a = e;
+      base += nt;
+      continue;
+    }
     if (base + nt > p.rows_cap) {  // only offsets that decrease give more tiles than the samples hold
       if (a == base && c.gt == 0) p.status[inst] = CROM_ERR_INVALID_ARG;
       a = e;
