@@ -20,6 +20,16 @@ static thread_local std::string g_last_error;
 
 void set_error(const std::string& msg) { g_last_error = msg; }
 
+cudaError_t clear_device(void* p, size_t bytes) {
+  cudaStream_t s;
+  cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(p, 0, bytes, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  const cudaError_t d = cudaStreamDestroy(s);
+  return e != cudaSuccess ? e : d;
+}
+
 namespace {
 
 int fail(int code, const std::string& msg) {

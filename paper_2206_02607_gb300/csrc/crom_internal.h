@@ -214,6 +214,27 @@ cudaError_t launch_step_fp32_noalloc(const crom_ctx* ctx, const crom_step_desc* 
                                      const float* samples, int n_samples, int max_samples, int* status,
                                      cudaStream_t s, size_t* need_bytes);
 
+// Clears device memory and returns once it is clear: a launch on any stream may use it
+// next.  (A plain cudaMemset runs on the legacy default stream, asynchronously to the
+// host, and a non-blocking stream is not ordered after it: a step on such a stream could
+// draw uncleared tickets.)  On a stream of its own, since a caller may be recording a
+// graph on its stream, and the default stream may have work queued.
+cudaError_t clear_device(void* p, size_t bytes);
+
+// Grows a scratch array of the context to n elements, all zero if `zero`.
+template <typename T>
+cudaError_t grow(crom_ctx* ctx, T** buf, size_t* cap, size_t n, bool zero = false) {
+  if (n <= *cap) return cudaSuccess;
+  if (*buf) cudaFree(*buf);
+  ++ctx->scratch_gen;
+  *buf = nullptr;
+  *cap = 0;
+  cudaError_t e = cudaMalloc(buf, n * sizeof(T));
+  if (e == cudaSuccess && zero) e = clear_device(*buf, n * sizeof(T));
+  if (e == cudaSuccess) *cap = n;
+  return e;
+}
+
 // Full-order model stencils (fom.cu).
 cudaError_t launch_fom(int kind, int n_batch, int nx, int ny, const float* coef, const float* ax, const float* ay,
                        double dt, int n_steps, float* u, float* tmp, cudaStream_t s);

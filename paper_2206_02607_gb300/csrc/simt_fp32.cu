@@ -875,60 +875,16 @@ cudaError_t launch_step_fp32(crom_ctx* ctx, const crom_step_desc* step, int n_in
   const int n_entries = r * (r + 1) / 2 + r;
 
   // Scratch: partial normal equations, per-instance tickets, per-sample targets.
-  const size_t need_part = (size_t)n_inst * max_tiles * n_entries;
-  if (need_part > ctx->partials_cap) {
-    if (ctx->partials) cudaFree(ctx->partials);
-    ++ctx->scratch_gen;
-    ctx->partials = nullptr;
-    ctx->partials_cap = 0;
-    cudaError_t e = cudaMalloc(&ctx->partials, need_part * sizeof(double));
-    if (e != cudaSuccess) return e;
-    ctx->partials_cap = need_part;
-  }
-  if ((size_t)n_inst > ctx->counters_cap) {
-    if (ctx->counters) cudaFree(ctx->counters);
-    ++ctx->scratch_gen;
-    ctx->counters = nullptr;
-    ctx->counters_cap = 0;
-    cudaError_t e = cudaMalloc(&ctx->counters, (size_t)n_inst * sizeof(int));
-    if (e != cudaSuccess) return e;
-    e = cudaMemset(ctx->counters, 0, (size_t)n_inst * sizeof(int));
-    if (e != cudaSuccess) return e;
-    ctx->counters_cap = n_inst;
-  }
-  // the chains of partial rows in groups (finish_cta): for few instances of many rows,
-  // whose last CTA would be alone with the sums
+  // The chains of partial rows go in groups (finish_cta) for few instances of many rows,
+  // whose last CTA would be alone with the sums.
   const int groups = kind == kFwdSmall && max_tiles > 16 ? kSumGroups : 1;
-  if (groups > 1 && (size_t)n_inst * groups > ctx->group_counters_cap) {
-    if (ctx->group_counters) cudaFree(ctx->group_counters);
-    ++ctx->scratch_gen;
-    ctx->group_counters = nullptr;
-    ctx->group_counters_cap = 0;
-    const size_t n = (size_t)n_inst * groups;
-    cudaError_t e = cudaMalloc(&ctx->group_counters, n * sizeof(int));
-    if (e != cudaSuccess) return e;
-    e = cudaMemset(ctx->group_counters, 0, n * sizeof(int));
-    if (e != cudaSuccess) return e;
-    ctx->group_counters_cap = n;
-  }
-  if ((size_t)n_samples > ctx->targets_cap) {
-    if (ctx->targets) cudaFree(ctx->targets);
-    ++ctx->scratch_gen;
-    ctx->targets = nullptr;
-    ctx->targets_cap = 0;
-    cudaError_t e = cudaMalloc(&ctx->targets, (size_t)n_samples * sizeof(double));
-    if (e != cudaSuccess) return e;
-    ctx->targets_cap = n_samples;
-  }
-  if ((size_t)n_inst * r > ctx->qbase_cap) {
-    if (ctx->qbase) cudaFree(ctx->qbase);
-    ++ctx->scratch_gen;
-    ctx->qbase = nullptr;
-    ctx->qbase_cap = 0;
-    cudaError_t e = cudaMalloc(&ctx->qbase, (size_t)n_inst * r * sizeof(double));
-    if (e != cudaSuccess) return e;
-    ctx->qbase_cap = (size_t)n_inst * r;
-  }
+  cudaError_t e = grow(ctx, &ctx->partials, &ctx->partials_cap, (size_t)n_inst * max_tiles * n_entries);
+  if (e == cudaSuccess) e = grow(ctx, &ctx->counters, &ctx->counters_cap, (size_t)n_inst, true);
+  if (e == cudaSuccess && groups > 1)
+    e = grow(ctx, &ctx->group_counters, &ctx->group_counters_cap, (size_t)n_inst * groups, true);
+  if (e == cudaSuccess) e = grow(ctx, &ctx->targets, &ctx->targets_cap, (size_t)n_samples);
+  if (e == cudaSuccess) e = grow(ctx, &ctx->qbase, &ctx->qbase_cap, (size_t)n_inst * r);
+  if (e != cudaSuccess) return e;
 
   p.S = S;
   p.off = s_off;
@@ -963,7 +919,7 @@ cudaError_t launch_step_fp32(crom_ctx* ctx, const crom_step_desc* step, int n_in
     p.second = (it == 0) ? kSecondLap : kSecondNone;
     p.nq = r;
     p.C = 1 + p.diff + ChannelSet{p.nx, p.second, p.nq}.count(m) - 1;
-    cudaError_t e = launch_fwd(p, kind, grid, s);
+    e = launch_fwd(p, kind, grid, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -1235,18 +1235,6 @@ size_t tc_step_smem_bytes(int img_bytes) {
 }
 
 namespace {
-// Grows a scratch array of the context to n elements.
-template <typename T>
-cudaError_t grow(crom_ctx* ctx, T** buf, size_t* cap, size_t n) {
-  if (n <= *cap) return cudaSuccess;
-  if (*buf) cudaFree(*buf);
-  ++ctx->scratch_gen;
-  *buf = nullptr;
-  *cap = 0;
-  const cudaError_t e = cudaMalloc(buf, n * sizeof(T));
-  if (e == cudaSuccess) *cap = n;
-  return e;
-}
 // Whether a step's iterations are launches of their own with the tiles dealt to all
 // groups, or one launch whose groups own whole instances.  In tiles per group: the split
 // iterations take about T / G (T tiles on G groups) and the cost of one tile more; the
@@ -1295,11 +1283,9 @@ cudaError_t launch_step_tc(crom_ctx* ctx, const crom_step_desc* step, int lo_par
   const bool split = step->line_search == 0 && !small_tiles && split_wanted(n_inst, n_samples, max_samples, tile, ctx->num_sms);
   if (split) {
     if ((e = grow(ctx, &ctx->partials, &ctx->partials_cap, ((size_t)n_samples / tile + n_inst) * n_entries)) != cudaSuccess ||
-        (e = grow(ctx, &ctx->qbase, &ctx->qbase_cap, (size_t)n_inst * ctx->desc.r)) != cudaSuccess)
+        (e = grow(ctx, &ctx->qbase, &ctx->qbase_cap, (size_t)n_inst * ctx->desc.r)) != cudaSuccess ||
+        (e = grow(ctx, &ctx->counters, &ctx->counters_cap, (size_t)n_inst, true)) != cudaSuccess)
       return e;
-    const size_t cap = ctx->counters_cap;
-    if ((e = grow(ctx, &ctx->counters, &ctx->counters_cap, (size_t)n_inst)) != cudaSuccess) return e;
-    if (ctx->counters_cap != cap && (e = cudaMemset(ctx->counters, 0, (size_t)n_inst * sizeof(int))) != cudaSuccess) return e;
   } else {
     order_kernel<<<1, 1024, 0, s>>>(s_off, n_inst, ctx->order, status, ctx->queue);
     e = cudaGetLastError();

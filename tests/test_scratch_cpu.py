@@ -1,0 +1,97 @@
+"""Host side of the context's and the trainer's scratch: what is cleared, allocated and
+freed before which launch, on a CUDA runtime without a device (fake_cudart.cpp, preloaded
+into a child process) that traces the calls.  No kernel runs."""
+import os
+import re
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+PRELUDE = """
+    import ctypes, os, sys
+    sys.path.insert(0, %r)
+    import numpy as np
+    from paper_2206_02607_gb300 import crom as c
+    from workloads import gen
+    fake = ctypes.CDLL(os.environ["LD_PRELOAD"])
+    fake.fake_limit.argtypes = [ctypes.c_size_t]
+    note = lambda t: fake.fake_note(t.encode())
+    S = 0x4440                       # a stream of the caller's, non-blocking
+    keep = []
+    def arr(a, t):
+        keep.append(np.ascontiguousarray(a, dtype=t))
+        return keep[-1].ctypes.data
+    def ok(rc):
+        assert rc == 0, (rc, c.last_error())
+    def context(m=2, r=8, width=128, hidden=5):
+        h, d = ctypes.c_void_p(), c.crom_decoder_desc(m, r, width, hidden)
+        ok(c.raw_call("crom_create", ctypes.byref(h), ctypes.byref(d), 0))
+        p = np.ascontiguousarray(gen.pack_params(gen.xavier_decoder(gen.DecoderSpec(m, r, width, hidden), seed=1)), np.float32)
+        keep.append(p)
+        ok(c.raw_call("crom_set_weights", h, p.ctypes.data, p.size, 0, S))
+        return h
+    def step(h, sizes, prec, gn=2, r=8, m=2, stream=S, status=0):
+        n, tot = len(sizes), int(sum(sizes))
+        sd = c.crom_step_desc(c.CROM_PDE_HEAT, gn, 1e-5)
+        rc = c.raw_call("crom_step", h, ctypes.byref(sd), prec, n, arr(np.zeros((n, r)), np.float64),
+                        arr(np.ones(n), np.float32), None, arr(gen.ragged_offsets(np.array(sizes)), np.int32),
+                        arr(np.zeros((tot, m)), np.float32), tot, max(sizes), arr(np.zeros(n), np.int32), stream)
+        assert rc == status, (rc, c.last_error())
+""" % ROOT
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    sys.path.insert(0, ROOT)
+    from paper_2206_02607_gb300 import build
+    from paper_2206_02607_gb300.build import _nvcc
+    build()
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_nvcc()))), "include")
+    so = str(tmp_path_factory.mktemp("fake") / "libfake_cudart.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", inc, os.path.join(HERE, "fake_cudart.cpp"), "-o", so,
+                    "-ldl"], check=True)
+    return so
+
+
+@pytest.fixture
+def trace(fake, tmp_path):
+    def run(body):
+        log = str(tmp_path / "trace")
+        env = dict(os.environ, LD_PRELOAD=fake, FAKE_CUDART_TRACE=log)
+        src = textwrap.dedent(PRELUDE) + textwrap.dedent(body)
+        res = subprocess.run([sys.executable, "-c", src], env=env, capture_output=True, text=True, timeout=300)
+        assert res.returncode == 0, res.stderr[-3000:]
+        with open(log) as f:
+            return f.read().splitlines()
+    return run
+
+
+def kernels(lines):
+    return [re.sub(r"^launch (\S+) .*", r"\1", x) for x in lines if x.startswith("launch ")]
+
+
+CLEARS = {
+    "fp32_few_samples": "step(context(), [200], c.CROM_PREC_FP32)",
+    "fp32_batch": "step(context(), [300] * 40, c.CROM_PREC_FP32)",
+    "dealt": "step(context(), [4096] * 8, c.CROM_PREC_F16X2)",
+    "whole": "step(context(), [64] * 1000, c.CROM_PREC_F16)",
+    "reconstruction": """
+        h = context()
+        ok(c.raw_call("crom_reconstruct", h, c.CROM_PREC_F16X2, 1, arr(np.zeros(8), np.float64), 4096,
+                      arr(np.zeros((4096, 2)), np.float32), arr(np.zeros(4096), np.float32), S))
+    """,
+}
+
+
+@pytest.mark.parametrize("case", sorted(CLEARS))
+def test_clears_and_copies_are_complete_before_the_first_launch(trace, case):
+    """The first call of a size on a non-blocking stream: every clear and copy that the
+    library made elsewhere is complete before a kernel of the call's stream can use it."""
+    lines = trace(CLEARS[case])
+    assert kernels(lines)
+    assert [x for x in lines if x.startswith("UNORDERED")] == []
