@@ -20,15 +20,17 @@ static thread_local std::string g_last_error;
 
 void set_error(const std::string& msg) { g_last_error = msg; }
 
-cudaError_t clear_device(void* p, size_t bytes) {
+static cudaError_t fill_device(void* p, const void* host, size_t bytes) {
   cudaStream_t s;
   cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(p, 0, bytes, s);
+  e = host ? cudaMemcpyAsync(p, host, bytes, cudaMemcpyHostToDevice, s) : cudaMemsetAsync(p, 0, bytes, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   const cudaError_t d = cudaStreamDestroy(s);
   return e != cudaSuccess ? e : d;
 }
+cudaError_t clear_device(void* p, size_t bytes) { return fill_device(p, nullptr, bytes); }
+cudaError_t upload_device(void* p, const void* host, size_t bytes) { return fill_device(p, host, bytes); }
 
 namespace {
 
@@ -922,9 +924,9 @@ int crom_trainer_load(crom_trainer* tr, const char* path) {
     return fail(CROM_ERR_INVALID_ARG, std::string(fn) + ": checksum mismatch in " + path);
   DeviceGuard g(tr->device);
   cudaError_t e = cudaDeviceSynchronize();
-  if (e == cudaSuccess) e = cudaMemcpy(tr->params, buf.data(), n * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(tr->am, buf.data() + n, n * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(tr->av, buf.data() + 2 * n, n * 4, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = upload_device(tr->params, buf.data(), n * 4);
+  if (e == cudaSuccess) e = upload_device(tr->am, buf.data() + n, n * 4);
+  if (e == cudaSuccess) e = upload_device(tr->av, buf.data() + 2 * n, n * 4);
   if (e != cudaSuccess) return cuda_fail(e, fn);
   tr->step = h.step;
   return CROM_OK;
@@ -983,8 +985,8 @@ int crom_trainer_set_params(crom_trainer* tr, const float* params, size_t n, int
                         "crom_trainer_set_params");
   if (st != CROM_OK) return st;
   DeviceGuard g(tr->device);
-  cudaError_t e = cudaMemset(tr->am, 0, n * 4);
-  if (e == cudaSuccess) e = cudaMemset(tr->av, 0, n * 4);
+  cudaError_t e = clear_device(tr->am, n * 4);
+  if (e == cudaSuccess) e = clear_device(tr->av, n * 4);
   if (e != cudaSuccess) return cuda_fail(e, "crom_trainer_set_params");
   tr->step = 0;
   return CROM_OK;

@@ -214,12 +214,14 @@ cudaError_t launch_step_fp32_noalloc(const crom_ctx* ctx, const crom_step_desc* 
                                      const float* samples, int n_samples, int max_samples, int* status,
                                      cudaStream_t s, size_t* need_bytes);
 
-// Clears device memory and returns once it is clear: a launch on any stream may use it
-// next.  (A plain cudaMemset runs on the legacy default stream, asynchronously to the
-// host, and a non-blocking stream is not ordered after it: a step on such a stream could
-// draw uncleared tickets.)  On a stream of its own, since a caller may be recording a
-// graph on its stream, and the default stream may have work queued.
+// Clear device memory, or fill it from pageable host memory, and return once that is
+// done: a launch on any stream may use it next.  (A plain cudaMemset or cudaMemcpy runs on
+// the legacy default stream and may still be under way when it returns, and a non-blocking
+// stream is not ordered after it: a step on such a stream could draw uncleared tickets.)
+// On a stream of its own, since a caller may be recording a graph on its stream, and the
+// default stream may have work queued.
 cudaError_t clear_device(void* p, size_t bytes);
+cudaError_t upload_device(void* p, const void* host, size_t bytes);
 
 // Grows a scratch array of the context to n elements, all zero if `zero`.
 template <typename T>

@@ -814,8 +814,8 @@ cudaError_t trainer_alloc(crom_trainer* t) {
   t->conv_part = (double*)A((t->lens.size() - 1) * kColChunks * 7 * 8);
   for (void* p : t->owned)
     if (!p) return cudaErrorMemoryAllocation;
-  cudaError_t e = cudaMemset(t->am, 0, o * 4);
-  if (e == cudaSuccess) e = cudaMemset(t->av, 0, o * 4);
+  cudaError_t e = clear_device(t->am, o * 4);
+  if (e == cudaSuccess) e = clear_device(t->av, o * 4);
   return e;
 }
 

@@ -391,8 +391,8 @@ cudaError_t trainer_tc_alloc(crom_trainer* t) {
   c.flag = (int*)A(sizeof(int));
   for (void* p : t->owned)
     if (!p) return cudaErrorMemoryAllocation;
-  cudaError_t e = cudaMemcpy(c.off_w, t->lay.dec_w.data(), (size_t)(L + 1) * sizeof(long), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemset(c.flag, 0, sizeof(int));
+  cudaError_t e = upload_device(c.off_w, t->lay.dec_w.data(), (size_t)(L + 1) * sizeof(long));
+  if (e == cudaSuccess) e = clear_device(c.flag, sizeof(int));
   if (e == cudaSuccess) c.ready = true;
   return e;
 }

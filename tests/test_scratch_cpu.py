@@ -85,6 +85,24 @@ CLEARS = {
         ok(c.raw_call("crom_reconstruct", h, c.CROM_PREC_F16X2, 1, arr(np.zeros(8), np.float64), 4096,
                       arr(np.zeros((4096, 2)), np.float32), arr(np.zeros(4096), np.float32), S))
     """,
+    "trainer": """
+        for prec in (c.CROM_PREC_FP32, c.CROM_PREC_BF16_MIXED):
+            for how in ("new", "set", "load"):
+                t, d = ctypes.c_void_p(), c.crom_decoder_desc(2, 8, 64, 3)
+                ok(c.raw_call("crom_trainer_create", ctypes.byref(t), ctypes.byref(d), 256, 2, 64, 0))
+                ok(c.raw_call("crom_trainer_set_precision", t, prec))
+                n = ctypes.c_size_t()
+                ok(c.raw_call("crom_trainer_param_count", t, ctypes.byref(n)))
+                p = arr(np.zeros(n.value), np.float32)
+                if how == "set":
+                    ok(c.raw_call("crom_trainer_set_params", t, p, n.value, 0, S))
+                if how == "load":
+                    path = (os.environ["FAKE_CUDART_TRACE"] + ".ckpt").encode()
+                    ok(c.raw_call("crom_trainer_save", t, path))
+                    ok(c.raw_call("crom_trainer_load", t, path))
+                ok(c.raw_call("crom_train_step", t, arr(np.zeros((2, 256)), np.float32), arr(np.zeros((2, 64)), np.int32),
+                              arr(np.zeros((256, 2)), np.float32), 1e-3, None, S))
+    """,
 }
 
 
