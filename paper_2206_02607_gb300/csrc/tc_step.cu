@@ -1067,7 +1067,6 @@ __global__ void __launch_bounds__(kThreads, 1) step_tc_kernel(StepParams p) {
   }
 
   if constexpr (kMode >= kIterFirst) {
-    if (kMode == kIterFirst && blockIdx.x == 0 && tid == 0) p.queue[1] = 0;  // the timeout flag
     ok = run_iteration<kM, kLoP, kMode>(c, p, own, Hbase, S->part, ok);
   }
   while (kMode < kIterFirst && ok) {
@@ -1286,6 +1285,8 @@ cudaError_t launch_step_tc(crom_ctx* ctx, const crom_step_desc* step, int lo_par
         (e = grow(ctx, &ctx->qbase, &ctx->qbase_cap, (size_t)n_inst * ctx->desc.r)) != cudaSuccess ||
         (e = grow(ctx, &ctx->counters, &ctx->counters_cap, (size_t)n_inst, true)) != cudaSuccess)
       return e;
+    // the timeout flag, before any CTA can set it
+    e = cudaMemsetAsync(ctx->queue + 1, 0, sizeof(int), s);
   } else {
     order_kernel<<<1, 1024, 0, s>>>(s_off, n_inst, ctx->order, status, ctx->queue);
     e = cudaGetLastError();

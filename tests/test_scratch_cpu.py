@@ -113,3 +113,22 @@ def test_clears_and_copies_are_complete_before_the_first_launch(trace, case):
     lines = trace(CLEARS[case])
     assert kernels(lines)
     assert [x for x in lines if x.startswith("UNORDERED")] == []
+
+
+@pytest.mark.parametrize("sizes", ["[4096] * 8", "[64] * 1000"])
+@pytest.mark.parametrize("prec", ["F16X2", "F16"])
+def test_the_timeout_flag_is_cleared_before_the_step_can_set_it(trace, sizes, prec):
+    """Dealt form (few instances): a clear of the flag on the step's stream, after the last
+    step's launches and before this one's first; whole form: the ordering kernel does it."""
+    lines = trace(f"""
+        h = context()
+        for k in range(2):
+            note("step")
+            step(h, {sizes}, c.CROM_PREC_{prec})
+    """)
+    flag = next(x for x in lines if x.startswith("malloc")).split()[1].split("+")[0] + "+4"  # the context's first array
+    for part in "\n".join(lines).split("\nstep\n")[1:]:
+        part = part.splitlines()
+        first = next(i for i, x in enumerate(part) if "step_tc_kernel" in x)
+        cleared = [x for x in part[:first] if x.startswith(f"memset {flag} 4 stream 0x4440")]
+        assert cleared or any("order_kernel" in x for x in part[:first]), part
