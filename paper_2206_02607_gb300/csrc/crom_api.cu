@@ -185,6 +185,10 @@ int crom_destroy(crom_ctx* ctx) {
     cudaFree(ctx->partials);
     cudaFree(ctx->counters);
     cudaFree(ctx->group_counters);
+    cudaFree(ctx->deal_rows);
+    cudaFree(ctx->deal_qbase);
+    cudaFree(ctx->deal_counters);
+    for (void* p : ctx->kept) cudaFree(p);
     cudaFree(ctx->targets);
     cudaFree(ctx->qbase);
     cudaFree(ctx->tangent);

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <algorithm>
 #include <vector>
 
 #include "../../include/crom.h"
@@ -73,12 +74,22 @@ struct crom_ctx {
   size_t partials_cap = 0;     // in doubles
   int* counters = nullptr;     // [n_inst], zero between launches
   size_t counters_cap = 0;
-  int* group_counters = nullptr;  // [n_inst][groups]: completed partial rows per group of chains, zero between launches
-  size_t group_counters_cap = 0;
   double* targets = nullptr;   // [n_samples]: Delta f_j (FP64) from GN iteration 0
   size_t targets_cap = 0;
   double* qbase = nullptr;     // [n_inst][r]: q_n kept for the difference channel
   size_t qbase_cap = 0;
+  // Scratch that some forms of a step take and others do not.  A larger one never frees a
+  // smaller one (grow_kept): a graph recorded with a step of one form stays valid whatever
+  // forms later steps within its sizes take.
+  int* group_counters = nullptr;  // [n_inst][groups]: completed partial rows per group of chains, zero between launches
+  size_t group_counters_cap = 0;
+  double* deal_rows = nullptr;    // dealt tiles: [tiles][n_entries], their normal-equation terms
+  size_t deal_rows_cap = 0;
+  double* deal_qbase = nullptr;   // [n_inst][r]: q_n
+  size_t deal_qbase_cap = 0;
+  int* deal_counters = nullptr;   // [n_inst]: tiles done, zero between launches
+  size_t deal_counters_cap = 0;
+  std::vector<void*> kept;        // smaller predecessors of the four, freed with the context
   float* tangent = nullptr;    // [n_inst][width]: layer-1 seeds W_1q qdot_i of the tangent velocity
   size_t tangent_cap = 0;
   uint8_t* host_stage = nullptr;  // crom_step_host: device copies of the caller's host arrays
@@ -235,6 +246,26 @@ cudaError_t grow(crom_ctx* ctx, T** buf, size_t* cap, size_t n, bool zero = fals
   if (e == cudaSuccess && zero) e = clear_device(*buf, n * sizeof(T));
   if (e == cudaSuccess) *cap = n;
   return e;
+}
+
+// The same for scratch that recorded graphs may go on using: the smaller array stays
+// allocated until the context is destroyed (capacities double, so these together are no
+// larger than the one in use).
+template <typename T>
+cudaError_t grow_kept(crom_ctx* ctx, T** buf, size_t* cap, size_t n, bool zero = false) {
+  if (n <= *cap) return cudaSuccess;
+  n = std::max(n, 2 * *cap);
+  T* p = nullptr;
+  cudaError_t e = cudaMalloc(&p, n * sizeof(T));
+  if (e == cudaSuccess && zero) e = clear_device(p, n * sizeof(T));
+  if (e != cudaSuccess) {
+    cudaFree(p);
+    return e;
+  }
+  if (*buf) ctx->kept.push_back(*buf);
+  *buf = p;
+  *cap = n;
+  return cudaSuccess;
 }
 
 // Full-order model stencils (fom.cu).

@@ -881,7 +881,7 @@ cudaError_t launch_step_fp32(crom_ctx* ctx, const crom_step_desc* step, int n_in
   cudaError_t e = grow(ctx, &ctx->partials, &ctx->partials_cap, (size_t)n_inst * max_tiles * n_entries);
   if (e == cudaSuccess) e = grow(ctx, &ctx->counters, &ctx->counters_cap, (size_t)n_inst, true);
   if (e == cudaSuccess && groups > 1)
-    e = grow(ctx, &ctx->group_counters, &ctx->group_counters_cap, (size_t)n_inst * groups, true);
+    e = grow_kept(ctx, &ctx->group_counters, &ctx->group_counters_cap, (size_t)n_inst * groups, true);
   if (e == cudaSuccess) e = grow(ctx, &ctx->targets, &ctx->targets_cap, (size_t)n_samples);
   if (e == cudaSuccess) e = grow(ctx, &ctx->qbase, &ctx->qbase_cap, (size_t)n_inst * r);
   if (e != cudaSuccess) return e;

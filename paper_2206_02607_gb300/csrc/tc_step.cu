@@ -1281,9 +1281,9 @@ cudaError_t launch_step_tc(crom_ctx* ctx, const crom_step_desc* step, int lo_par
   const int tile = lo_parts ? kLarge : 2 * kLarge, n_entries = ctx->desc.r * (ctx->desc.r + 3) / 2;
   const bool split = step->line_search == 0 && !small_tiles && split_wanted(n_inst, n_samples, max_samples, tile, ctx->num_sms);
   if (split) {
-    if ((e = grow(ctx, &ctx->partials, &ctx->partials_cap, ((size_t)n_samples / tile + n_inst) * n_entries)) != cudaSuccess ||
-        (e = grow(ctx, &ctx->qbase, &ctx->qbase_cap, (size_t)n_inst * ctx->desc.r)) != cudaSuccess ||
-        (e = grow(ctx, &ctx->counters, &ctx->counters_cap, (size_t)n_inst, true)) != cudaSuccess)
+    if ((e = grow_kept(ctx, &ctx->deal_rows, &ctx->deal_rows_cap, ((size_t)n_samples / tile + n_inst) * n_entries)) != cudaSuccess ||
+        (e = grow_kept(ctx, &ctx->deal_qbase, &ctx->deal_qbase_cap, (size_t)n_inst * ctx->desc.r)) != cudaSuccess ||
+        (e = grow_kept(ctx, &ctx->deal_counters, &ctx->deal_counters_cap, (size_t)n_inst, true)) != cudaSuccess)
       return e;
     // the timeout flag, before any CTA can set it
     e = cudaMemsetAsync(ctx->queue + 1, 0, sizeof(int), s);
@@ -1324,10 +1324,10 @@ cudaError_t launch_step_tc(crom_ctx* ctx, const crom_step_desc* step, int lo_par
   p.order = ctx->order;
   p.queue = ctx->queue;
   p.df = ctx->targets;
-  p.qbase = ctx->qbase;
-  p.rows = ctx->partials;
+  p.qbase = ctx->deal_qbase;
+  p.rows = ctx->deal_rows;
   p.rows_cap = n_samples / tile + n_inst;
-  p.counters = ctx->counters;
+  p.counters = ctx->deal_counters;
   const size_t smem = tc_step_smem_bytes(p.img_bytes);
   const int grid = split ? (int)std::min<long long>((long long)n_samples / tile + n_inst, ctx->num_sms)
                          : std::min((n_inst + kGroups - 1) / kGroups, ctx->num_sms);

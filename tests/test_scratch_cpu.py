@@ -132,3 +132,26 @@ def test_the_timeout_flag_is_cleared_before_the_step_can_set_it(trace, sizes, pr
         first = next(i for i, x in enumerate(part) if "step_tc_kernel" in x)
         cleared = [x for x in part[:first] if x.startswith(f"memset {flag} 4 stream 0x4440")]
         assert cleared or any("order_kernel" in x for x in part[:first]), part
+
+
+STEADY = {
+    "dealt_after_whole": ["step(h, [64] * 1000, c.CROM_PREC_F16X2)", "step(h, [1000] * 8, c.CROM_PREC_F16)",
+                          "step(h, [1000] * 8, c.CROM_PREC_F16X2)", "step(h, [6000] * 10, c.CROM_PREC_F16X2)"],
+    "dealt_after_fp32": ["step(h, [10000], c.CROM_PREC_FP32)", "step(h, [64] * 20, c.CROM_PREC_F16X2, gn=1)",
+                         "step(h, [1000] * 8, c.CROM_PREC_F16X2)"],
+    "few_samples_fp32": ["step(h, [64] * 1000, c.CROM_PREC_FP32)", "step(h, [200], c.CROM_PREC_FP32)",
+                         "step(h, [100] * 3, c.CROM_PREC_FP32)"],
+}
+
+
+@pytest.mark.parametrize("case", sorted(STEADY))
+def test_steps_within_earlier_sizes_free_nothing(trace, case):
+    """Once a context has stepped a batch of the largest sizes, smaller steps free no
+    array, whatever form they take: a graph recorded with any of them stays valid."""
+    first, *rest = STEADY[case]
+    body = ["h = context()", first, 'note("steady")'] + rest + ['note("end")', 'ok(c.raw_call("crom_destroy", h))']
+    lines = trace("\n".join(body))
+    a, b = lines.index("steady"), lines.index("end")
+    assert [x for x in lines[a:b] if x.startswith("free")] == []
+    made = {x.split()[1] for x in lines if x.startswith("malloc #")}
+    assert made == {x.split()[1] for x in lines if x.startswith("free #")}      # all given back
