@@ -268,6 +268,29 @@ cudaError_t grow_kept(crom_ctx* ctx, T** buf, size_t* cap, size_t n, bool zero =
   return cudaSuccess;
 }
 
+// grow_kept for scratch that a call can do without: *have says whether the array holds n
+// elements now.  It does not grow while the caller records a graph on s (an allocation
+// could end the recording; the library's own recording allows it), nor when the device is
+// out of memory.
+template <typename T>
+cudaError_t try_grow_kept(crom_ctx* ctx, cudaStream_t s, T** buf, size_t* cap, size_t n, bool zero, bool* have) {
+  *have = n <= *cap;
+  if (*have) return cudaSuccess;
+  cudaStreamCaptureStatus recording = cudaStreamCaptureStatusNone;
+  if (s == nullptr || s != ctx->cap_stream) {
+    if (cudaStreamIsCapturing(s, &recording) != cudaSuccess) recording = cudaStreamCaptureStatusActive;
+  }
+  if (recording != cudaStreamCaptureStatusNone) {
+    (void)cudaGetLastError();
+    return cudaSuccess;
+  }
+  const cudaError_t e = grow_kept(ctx, buf, cap, n, zero);
+  *have = e == cudaSuccess;
+  if (e != cudaErrorMemoryAllocation) return e;
+  (void)cudaGetLastError();
+  return cudaSuccess;
+}
+
 // Full-order model stencils (fom.cu).
 cudaError_t launch_fom(int kind, int n_batch, int nx, int ny, const float* coef, const float* ax, const float* ay,
                        double dt, int n_steps, float* u, float* tmp, cudaStream_t s);

@@ -877,11 +877,14 @@ cudaError_t launch_step_fp32(crom_ctx* ctx, const crom_step_desc* step, int n_in
   // Scratch: partial normal equations, per-instance tickets, per-sample targets.
   // The chains of partial rows go in groups (finish_cta) for few instances of many rows,
   // whose last CTA would be alone with the sums.
-  const int groups = kind == kFwdSmall && max_tiles > 16 ? kSumGroups : 1;
+  int groups = kind == kFwdSmall && max_tiles > 16 ? kSumGroups : 1;
   cudaError_t e = grow(ctx, &ctx->partials, &ctx->partials_cap, (size_t)n_inst * max_tiles * n_entries);
   if (e == cudaSuccess) e = grow(ctx, &ctx->counters, &ctx->counters_cap, (size_t)n_inst, true);
-  if (e == cudaSuccess && groups > 1)
-    e = grow_kept(ctx, &ctx->group_counters, &ctx->group_counters_cap, (size_t)n_inst * groups, true);
+  if (e == cudaSuccess && groups > 1) {  // the same sums without them
+    bool have;
+    e = try_grow_kept(ctx, s, &ctx->group_counters, &ctx->group_counters_cap, (size_t)n_inst * groups, true, &have);
+    if (!have) groups = 1;
+  }
   if (e == cudaSuccess) e = grow(ctx, &ctx->targets, &ctx->targets_cap, (size_t)n_samples);
   if (e == cudaSuccess) e = grow(ctx, &ctx->qbase, &ctx->qbase_cap, (size_t)n_inst * r);
   if (e != cudaSuccess) return e;

@@ -1277,14 +1277,16 @@ cudaError_t launch_step_tc(crom_ctx* ctx, const crom_step_desc* step, int lo_par
   constexpr int kLarge = kTcTileS1Large, kSmall = kTcTileS1Small;
   const bool small_tiles = ctx->tc_tile_s1 == kSmall;
   // Split mode: see split_wanted.  Its tile rows are sized for every instance's ragged
-  // last tile.
+  // last tile; without them the groups take whole instances, which gives the same bits.
   const int tile = lo_parts ? kLarge : 2 * kLarge, n_entries = ctx->desc.r * (ctx->desc.r + 3) / 2;
-  const bool split = step->line_search == 0 && !small_tiles && split_wanted(n_inst, n_samples, max_samples, tile, ctx->num_sms);
+  bool split = step->line_search == 0 && !small_tiles && split_wanted(n_inst, n_samples, max_samples, tile, ctx->num_sms);
+  if (split)
+    e = try_grow_kept(ctx, s, &ctx->deal_rows, &ctx->deal_rows_cap, ((size_t)n_samples / tile + n_inst) * n_entries, false, &split);
+  if (split)
+    e = try_grow_kept(ctx, s, &ctx->deal_qbase, &ctx->deal_qbase_cap, (size_t)n_inst * ctx->desc.r, false, &split);
+  if (split) e = try_grow_kept(ctx, s, &ctx->deal_counters, &ctx->deal_counters_cap, (size_t)n_inst, true, &split);
+  if (e != cudaSuccess) return e;
   if (split) {
-    if ((e = grow_kept(ctx, &ctx->deal_rows, &ctx->deal_rows_cap, ((size_t)n_samples / tile + n_inst) * n_entries)) != cudaSuccess ||
-        (e = grow_kept(ctx, &ctx->deal_qbase, &ctx->deal_qbase_cap, (size_t)n_inst * ctx->desc.r)) != cudaSuccess ||
-        (e = grow_kept(ctx, &ctx->deal_counters, &ctx->deal_counters_cap, (size_t)n_inst, true)) != cudaSuccess)
-      return e;
     // the timeout flag, before any CTA can set it
     e = cudaMemsetAsync(ctx->queue + 1, 0, sizeof(int), s);
   } else {

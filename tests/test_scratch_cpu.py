@@ -155,3 +155,38 @@ def test_steps_within_earlier_sizes_free_nothing(trace, case):
     assert [x for x in lines[a:b] if x.startswith("free")] == []
     made = {x.split()[1] for x in lines if x.startswith("malloc #")}
     assert made == {x.split()[1] for x in lines if x.startswith("free #")}      # all given back
+
+
+def test_a_step_without_room_for_its_rows_takes_the_whole_form(trace):
+    """Where the dealt form's rows cannot be allocated, the groups take whole instances
+    (which need 8 bytes a sample); with room again, the step is dealt."""
+    lines = trace("""
+        h = context()
+        fake.fake_limit(500000)          # the targets take 262144 bytes, the rows 723712
+        step(h, [4096] * 8, c.CROM_PREC_F16X2)
+        note("room")
+        fake.fake_limit(1 << 40)
+        step(h, [4096] * 8, c.CROM_PREC_F16X2)
+    """)
+    a = lines.index("room")
+    assert any(x.startswith("malloc refused 723712") for x in lines[:a])
+    assert [("order" in k) for k in kernels(lines[:a])] == [True, False]
+    assert [("order" in k) for k in kernels(lines[a:])] == [False, False]
+
+
+@pytest.mark.parametrize("warm,call,whole", [("[64] * 1000, c.CROM_PREC_F16X2", "[1000] * 8, c.CROM_PREC_F16X2", True),
+                                             ("[64] * 1000, c.CROM_PREC_FP32", "[200], c.CROM_PREC_FP32", False)])
+def test_a_recorded_step_within_earlier_sizes_allocates_nothing(trace, warm, call, whole):
+    """While the caller records its stream, a step within the sizes of an earlier one
+    allocates nothing, although its form has not run before."""
+    lines = trace(f"""
+        h = context()
+        step(h, {warm})
+        note("recording")
+        fake.fake_capturing(1)
+        step(h, {call})
+        fake.fake_capturing(0)
+    """)
+    part = lines[lines.index("recording"):]
+    assert not any("malloc" in x for x in part), part
+    assert len(kernels(part)) == 2 and ("order" in kernels(part)[0]) == whole
