@@ -230,7 +230,8 @@ int crom_device_flags(crom_ctx* ctx, int* flags, crom_stream stream);
  * (paper Algorithm 3).  Instance i has latent state q[i] (FP64 [n_inst][r],
  * updated in place), coefficient alpha[i] (FP32), and integration samples
  * samples[s_off[i] .. s_off[i+1]) (FP32 [n_samples][m]; s_off int32
- * [n_inst+1], s_off[0] = 0, s_off[n_inst] = n_samples).  vel (FP32
+ * [n_inst+1], s_off[0] = 0, s_off[n_inst] = n_samples; ranges may overlap only with
+ * gn_iters == 1, as later iterations keep Delta f per sample).  vel (FP32
  * [n_samples][m]) is the advection velocity at each sample, required for
  * CROM_PDE_ADVDIFF and ignored (may be NULL) otherwise.  max_samples must bound
  * every |M_i|; an instance with |M_i| > max_samples or |M_i| < r gets

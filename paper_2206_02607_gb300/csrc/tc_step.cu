@@ -126,7 +126,7 @@ struct StepParams {
   // split mode (kIterFirst, kIterLater): one launch per Gauss-Newton iteration
   double* qbase;   // [n_inst][r]: q_n, written by iteration 0's solve
   double* rows;    // [tiles][entries]: every tile's normal-equation terms
-  int rows_cap;    // tiles that rows holds
+  int rows_cap;    // tiles that rows holds; two more rows per group follow
   int* counters;   // [n_inst]: tiles done, zero between launches
 };
 // What an instantiation of the kernel does: whole steps (instances from a queue), Step 1
@@ -891,15 +891,13 @@ __device__ __forceinline__ bool run_iteration(Lane& c, const StepParams& p, Own&
   for (; a < b; ++inst) {
     const int nt = deal_tiles<kSS>(p, inst);
     if (nt == 0) continue;
-    const int e = min(b, base + nt), o0 = p.off[inst], M = p.off[inst + 1] - o0;
-    if (kMode == kIterLater && p.status[inst] != CROM_OK) {
-      a = e;
-      base += nt;
-      continue;
-    }
-    if (base + nt > p.rows_cap) {  // only offsets that decrease give more tiles than the samples hold
-      if (a == base && c.gt == 0) p.status[inst] = CROM_ERR_INVALID_ARG;
-      a = e;
+    // Rows for the tiles of n_samples samples: only offsets that decrease (ranges that
+    // overlap) give more.  The group with such an instance's first tile takes all of it,
+    // through two rows of its own (a tile's terms and their sum).
+    const bool alone = base + nt > p.rows_cap;
+    const int e = alone && a == base ? base + nt : min(b, base + nt), o0 = p.off[inst], M = p.off[inst + 1] - o0;
+    if ((alone && a != base) || (kMode == kIterLater && p.status[inst] != CROM_OK)) {
+      a = min(b, e);
       base += nt;
       continue;
     }
@@ -914,10 +912,14 @@ __device__ __forceinline__ bool run_iteration(Lane& c, const StepParams& p, Own&
       const float alpha = p.coef_per_sample ? 0.f : p.alpha[inst];
       set_layer1<kM>(c, p, G, G->qcur);
       for (int t = a - base; t < e - base && ok; ++t) {
-        own.row = p.rows + (size_t)(base + t) * n_entries;
+        own.row = p.rows + (size_t)(alone ? p.rows_cap + 2 * gid : base + t) * n_entries;
         const int ns = min(kSS, M - t * kSS);
         if constexpr (kMode == kIterFirst) ok = run_pair<kM, kLoP, kMode>(c, p, o0, t, ns, alpha, own);
         else ok = run_tile<kM, kSS, kLoP, kMode>(c, p, o0, t, ns, alpha, own);
+        if (alone) {
+          for (int k = c.gt; k < n_entries; k += kGT)  // a thread's own entries
+            own.row[n_entries + k] = own.row[k] + (t > 0 ? own.row[n_entries + k] : 0.0);
+        }
       }
     }
     group_sync(c.g);  // every thread's terms are written
@@ -937,16 +939,17 @@ __device__ __forceinline__ bool run_iteration(Lane& c, const StepParams& p, Own&
         for (int k = 0; k < 2; ++k) {
           const int ea = own.ea[k], eb = own.eb[k];
           if (ea < 0) continue;
-          const double* x = p.rows + (size_t)base * n_entries + c.gt + k * kGT;
+          const double* x = p.rows + (size_t)(alone ? p.rows_cap + 2 * gid + 1 : base) * n_entries + c.gt + k * kGT;
+          const int n = alone ? 1 : nt;
           double acc = 0.0;
-          for (int t0 = 0; t0 < nt; t0 += 16) {  // loads ahead of the additions
+          for (int t0 = 0; t0 < n; t0 += 16) {  // loads ahead of the additions
             double v[16];
 #pragma unroll
             for (int t = 0; t < 16; ++t)
-              if (t0 + t < nt) v[t] = __ldcg(x + (size_t)(t0 + t) * n_entries);
+              if (t0 + t < n) v[t] = __ldcg(x + (size_t)(t0 + t) * n_entries);
 #pragma unroll
             for (int t = 0; t < 16; ++t)
-              if (t0 + t < nt) acc += v[t];
+              if (t0 + t < n) acc += v[t];
           }
           if (eb >= 0) {
             G->amat[ea * R + eb] = acc;
@@ -1244,7 +1247,8 @@ namespace {
 // Far above one instance per group only the caller's bound on |M_i| could ask for it.
 bool split_wanted(int n_inst, int n_samples, int max_samples, int tile, int num_sms) {
   const double G = kGroups * num_sms;
-  if (n_inst > 1.25 * G) return false;
+  // (the prefix sums of the tiles are 32-bit, whatever the offsets)
+  if (n_inst > 1.25 * G || ceil((double)std::min(max_samples, n_samples) / tile) * n_inst >= 2147483648.0) return false;
   const double mean = (double)n_samples / n_inst / tile, T = (mean + 0.5) * n_inst;
   const double largest = ceil((double)std::min(max_samples, n_samples) / tile);
   const double whole = largest <= 1.25 * mean ? std::max(largest, ceil(n_inst / G) * mean) : largest;
@@ -1280,8 +1284,10 @@ cudaError_t launch_step_tc(crom_ctx* ctx, const crom_step_desc* step, int lo_par
   // last tile; without them the groups take whole instances, which gives the same bits.
   const int tile = lo_parts ? kLarge : 2 * kLarge, n_entries = ctx->desc.r * (ctx->desc.r + 3) / 2;
   bool split = step->line_search == 0 && !small_tiles && split_wanted(n_inst, n_samples, max_samples, tile, ctx->num_sms);
+  const int tile_rows = n_samples / tile + n_inst, deal_grid = std::min(tile_rows, ctx->num_sms);
   if (split)
-    e = try_grow_kept(ctx, s, &ctx->deal_rows, &ctx->deal_rows_cap, ((size_t)n_samples / tile + n_inst) * n_entries, false, &split);
+    e = try_grow_kept(ctx, s, &ctx->deal_rows, &ctx->deal_rows_cap,
+                      ((size_t)tile_rows + 2 * kGroups * deal_grid) * n_entries, false, &split);
   if (split)
     e = try_grow_kept(ctx, s, &ctx->deal_qbase, &ctx->deal_qbase_cap, (size_t)n_inst * ctx->desc.r, false, &split);
   if (split) e = try_grow_kept(ctx, s, &ctx->deal_counters, &ctx->deal_counters_cap, (size_t)n_inst, true, &split);
@@ -1328,11 +1334,10 @@ cudaError_t launch_step_tc(crom_ctx* ctx, const crom_step_desc* step, int lo_par
   p.df = ctx->targets;
   p.qbase = ctx->deal_qbase;
   p.rows = ctx->deal_rows;
-  p.rows_cap = n_samples / tile + n_inst;
+  p.rows_cap = tile_rows;
   p.counters = ctx->deal_counters;
   const size_t smem = tc_step_smem_bytes(p.img_bytes);
-  const int grid = split ? (int)std::min<long long>((long long)n_samples / tile + n_inst, ctx->num_sms)
-                         : std::min((n_inst + kGroups - 1) / kGroups, ctx->num_sms);
+  const int grid = split ? deal_grid : std::min((n_inst + kGroups - 1) / kGroups, ctx->num_sms);
   auto launch = [&](auto kernel) -> cudaError_t {
     cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;

@@ -102,3 +102,36 @@ def test_failure_after_the_first_iteration(c, prec_name, gn):
         fresh_ctx.close()
     ctx.close()
     other.close()
+
+
+@pytest.mark.parametrize("prec_name", ["CROM_PREC_F16X2", "CROM_PREC_F16"])
+def test_overlapping_sample_ranges(c, prec_name):
+    """Offsets that decrease between instances whose ranges overlap: the instances in
+    between are refused, the others give the bits they give on their own, though their
+    tiles are more than the samples make.  One Gauss-Newton iteration: later ones keep
+    Delta f per sample, which overlapping instances share in every form of the step."""
+    import torch
+    prec, n = getattr(c, prec_name), 400
+    params = gen.xavier_decoder(gen.DecoderSpec(2, 8, 128, 4), seed=3, bias_std=0.1)
+    ctx = _ctx(c, params, 4)
+    rng = np.random.default_rng(11)
+    x = rng.uniform(0, 1, size=(n, 2)).astype(np.float32)
+    off = np.array([0, 300, 100, 400, 0, 400, 0, 17, 1, 400])
+    k = len(off) - 1
+    q, alpha = rng.standard_normal((k, 8)), rng.uniform(0.5, 2.0, size=k).astype(np.float32)
+    qd, st = dev(q, torch.float64), torch.full((k,), -1, dtype=torch.int32, device="cuda")
+    for _ in range(2):
+        c.crom_step(ctx, qd, dev(alpha, torch.float32), dev(off, torch.int32), dev(x, torch.float32), st, dt=1e-5,
+                    gn_iters=1, max_samples=n, precision=prec)
+    got, st = qd.cpu().numpy(), st.cpu().numpy()
+    for i in range(k):
+        lo, hi = off[i], off[i + 1]
+        if hi < lo:
+            assert st[i] == c.CROM_ERR_INVALID_ARG and np.array_equal(got[i], q[i]), i
+            continue
+        one = Batch(np.array([hi - lo]), x[lo:hi], q[i:i + 1], alpha[i:i + 1])
+        for _ in range(2):
+            one.step(c, ctx, prec, 1)
+        want, st_want = one.result()
+        assert st[i] == st_want[0] == c.CROM_OK and np.array_equal(got[i], want[0]), i
+    ctx.close()
