@@ -18,6 +18,7 @@
 //    kFieldMaxAdv): one CTA per field, the field twice in shared memory, one barrier per
 //    step (100 steps of 256 nodes: 409 -> 14 us; 10 steps of 97^2, heat: 41 -> 24 us).
 #include <algorithm>
+#include <atomic>
 
 #include "crom_internal.h"
 
@@ -415,7 +416,7 @@ __global__ void __launch_bounds__(1024) fom_line_kernel(float* u, const float* c
 // 97, growing with the area, against 4.1 us for a launch per step: the largest sides.
 constexpr int kFieldMaxHeat = 128, kFieldMaxAdv = 100;
 template <int kScheme>
-__global__ void __launch_bounds__(1024) fom_field_kernel(FomParams p) {
+__device__ __forceinline__ void fom_field_body(const FomParams& p) {
   constexpr bool kAdv = kScheme >= kUpwind, kCen = kScheme == kCentral;
   extern __shared__ float4 smem4[];
   const int n = p.n, N = n * n, NT = blockDim.x;
@@ -467,6 +468,47 @@ __global__ void __launch_bounds__(1024) fom_field_kernel(FomParams p) {
   }
   for (int e = threadIdx.x; e < N; e += blockDim.x) p.u[base + e] = src[e];
 }
+// Two CTAs on an SM for many fields: 3000 fields of 57^2, heat, one step, 67 us with one,
+// 48 with two.  The heat form spills 28 bytes for it (one field of 49^2, 20 steps: 15
+// against 19 us), so few fields take the one without the bound.
+template <int kScheme>
+__global__ void __launch_bounds__(1024, 2) fom_field_kernel(FomParams p) { fom_field_body<kScheme>(p); }
+__global__ void __launch_bounds__(1024) fom_field_few_kernel(FomParams p) { fom_field_body<kHeat>(p); }
+
+// Whether one launch of fom_field_kernel pays against a launch per step, in microseconds
+// as measured over sides 49 to 127, 1 to 3000 fields and 1 to 50 steps (with these lines
+// no shape is more than 4 % slower than a launch per step).
+//  * Fewer fields than SMs: the launch takes 9 and, per step, 3.0 (heat), 3.75 (with a
+//    coefficient field) or 4.7 (advection) at side 127 in proportion to the area; a launch
+//    per step 4.2 (more where the fields' bytes take longer; an odd count copies back as
+//    long as a step), a call at least 13.  Ten fields of 127^2 with a coefficient field,
+//    four steps: 26 against 18 us; 20 steps: 85 against 84; of 97^2, eight: 26 against 35.
+//  * Heat from side 120 on (one field an SM), one or two steps of many fields: the loads
+//    are not overlapped.  1000 with a coefficient field, 127^2, one step: 115 against 87
+//    us, two 141 against 121; 3000 of heat 266 against 225.
+bool field_pays(int scheme, int n, int n_batch, int steps, int sms) {
+  const double nodes = (double)n * n;
+  if (n_batch < sms) {
+    const double per_step = (scheme == kHeat ? 3.0 : scheme == kHeatField ? 3.75 : 4.7) * nodes / (127 * 127);
+    const double launch = std::max(4.2, 3.3 + (scheme >= kUpwind ? 8e-6 : 3.5e-6) * n_batch * nodes);
+    return 9.0 + steps * per_step <= std::max(13.0, (steps + (steps & 1)) * launch);
+  }
+  return scheme >= kUpwind || n < 120 || steps > 2 || n_batch <= (scheme == kHeatField ? 4 : 12) * sms;
+}
+
+// SMs of the current device.  Asked for once per device: the attribute query took 0.7 us
+// of each call, 5 % of one with a launch or two.
+cudaError_t sm_count(int* sms) {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  *sms = dev < 64 ? known[dev].load(std::memory_order_relaxed) : 0;
+  if (*sms > 0) return cudaSuccess;
+  e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess && dev < 64) known[dev].store(*sms, std::memory_order_relaxed);
+  return e;
+}
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
@@ -492,9 +534,8 @@ template <int kScheme>
 cudaError_t launch_2d(const FomParams& p, int n_batch, cudaStream_t s, bool* done) {
   const int n = p.n;
   const bool field = kScheme == kHeatField, adv = kScheme >= kUpwind;
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
   // One or two steps of a batch that streams through HBM gain nothing from staying on
   // the chip, and the velocities' load is not overlapped there: 512 fields of 256^2, one
@@ -515,6 +556,14 @@ cudaError_t launch_2d(const FomParams& p, int n_batch, cudaStream_t s, bool* don
       if (n == 128) return launch_cluster(fom_wide_kernel<kScheme, 32>, p, 1, n_batch, kWideThreads, wide_bytes<kScheme, 32>(), s);
       return launch_cluster(fom_wide_kernel<kScheme, 64>, p, 4, n_batch, kWideThreads, wide_bytes<kScheme, 64>(), s);
     }
+    // One step by clusters of eight CTAs, the GPU full: the loads and stores of such a call
+    // are not overlapped.  Sides 180 to 192 leave 288 threads a CTA: 600 fields of 180^2,
+    // heat with a coefficient field, 115 against 107 us.  Advection: 300 fields of 212^2 88
+    // against 84 us, of 180^2 74 (two steps 95) against 63 (92); up to 200 fields no slower.
+    const int thr = tile_thr(n, RT, NC);
+    if (NC == 8 && ((adv && 2 * n_batch > 3 * sms && p.steps <= (thr <= 288 ? 2 : 1)) ||
+                    (field && thr <= 288 && n_batch >= sms && p.steps == 1)))
+      return cudaSuccess;
     if ((long long)n_batch * NC < sms) {
       while (n > 64 && NC < 8 && (long long)n_batch * NC * 2 <= sms) NC *= 2;
       while (RT > 1 && tile_thr(n, RT / 2, NC) <= (NC > 1 ? 256 : kTileThreads)) RT /= 2;
@@ -528,12 +577,13 @@ cudaError_t launch_2d(const FomParams& p, int n_batch, cudaStream_t s, bool* don
     }
   }
   // (two steps of advection at side 97: 14.5 us against 13.8 us for two launches)
-  if (n <= (adv ? kFieldMaxAdv : kFieldMaxHeat) && (!adv || p.steps > 2)) {
+  if (n <= (adv ? kFieldMaxAdv : kFieldMaxHeat) && (!adv || p.steps > 2) && field_pays(kScheme, n, n_batch, p.steps, sms)) {
     const size_t smem = (size_t)(adv ? 4 : 2) * n * n * sizeof(float);
-    e = cudaFuncSetAttribute(fom_field_kernel<kScheme>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const auto kernel = kScheme == kHeat && n_batch <= sms ? fom_field_few_kernel : fom_field_kernel<kScheme>;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     *done = true;
-    fom_field_kernel<kScheme><<<n_batch, std::min(1024, (n * n + 31) / 32 * 32), smem, s>>>(p);
+    kernel<<<n_batch, std::min(1024, (n * n + 31) / 32 * 32), smem, s>>>(p);
     return cudaGetLastError();
   }
   return cudaSuccess;
@@ -546,6 +596,15 @@ cudaError_t launch_fom_fused(int kind, int n_batch, int nx, const float* coef, c
   *done = false;
   if (kind == CROM_FOM_HEAT1D_DIRICHLET || kind == CROM_FOM_HEAT1D_DIRICHLET_FIELD) {
     if (nx > kLineMax) return cudaSuccess;
+    // One or two steps of many short lines: a CTA per line does not overlap its load, step
+    // and store.  16000 lines of 1500 with a coefficient field, one step: 155 against 117
+    // us; 8000 of 700, two: 38 against 34; without, 8000 of 1024, one: 33 against 31 (16000,
+    // which no longer stay in L2 with their copies: 61 against 77).
+    const long long nodes = (long long)n_batch * nx;
+    const bool short_lines = kind == CROM_FOM_HEAT1D_DIRICHLET_FIELD
+                                 ? (n_steps == 1 && nx <= 4096) || (n_steps == 2 && nx < 2048)
+                                 : n_steps == 1 && nx <= 1024 && nodes < 12000000;
+    if (nodes > 5000000 && short_lines) return cudaSuccess;
     const double dx = 1.0 / (nx - 1);
     const float r_over = (float)(dt / (dx * dx));
     const size_t smem = (size_t)2 * nx * sizeof(float);

@@ -190,3 +190,32 @@ def test_a_recorded_step_within_earlier_sizes_allocates_nothing(trace, warm, cal
     part = lines[lines.index("recording"):]
     assert not any("malloc" in x for x in part), part
     assert len(kernels(part)) == 2 and ("order" in kernels(part)[0]) == whole
+
+
+# kind, side, ny, fields, steps, whether the steps are one launch: shapes at which the one
+# launch was measured slower than a launch per step (False), and their neighbours
+FOM_ROUTES = [("HEAT2D_NEUMANN_FIELD", 127, 10, 4, False), ("HEAT2D_NEUMANN_FIELD", 127, 10, 50, True),
+              ("HEAT2D_NEUMANN", 121, 1, 4, False), ("HEAT2D_NEUMANN", 121, 1, 12, True),
+              ("HEAT2D_NEUMANN", 97, 10, 8, True), ("ADVDIFF2D_PERIODIC", 99, 10, 4, False),
+              ("ADVDIFF2D_PERIODIC_CENTRAL", 97, 10, 8, True), ("HEAT2D_NEUMANN_FIELD", 125, 1000, 1, False),
+              ("HEAT2D_NEUMANN_FIELD", 125, 1000, 3, True), ("HEAT2D_NEUMANN", 127, 3000, 1, False),
+              ("HEAT2D_NEUMANN", 117, 3000, 1, True), ("ADVDIFF2D_PERIODIC", 180, 300, 1, False),
+              ("ADVDIFF2D_PERIODIC", 180, 300, 3, True), ("ADVDIFF2D_PERIODIC", 164, 300, 1, True),
+              ("HEAT2D_NEUMANN_FIELD", 180, 600, 1, False), ("HEAT2D_NEUMANN_FIELD", 212, 600, 1, True),
+              ("HEAT1D_DIRICHLET_FIELD", 1500, 16000, 1, False), ("HEAT1D_DIRICHLET_FIELD", 700, 8000, 2, False),
+              ("HEAT1D_DIRICHLET_FIELD", 1500, 16000, 3, True), ("HEAT1D_DIRICHLET", 1024, 8000, 1, False),
+              ("HEAT1D_DIRICHLET", 1024, 16000, 1, True)]
+
+
+def test_full_order_steps_take_the_faster_launches(trace):
+    body = "p = 0x7f0000000000          # not read: no kernel runs\n"
+    for kind, n, nb, steps, _ in FOM_ROUTES:
+        two_d = not kind.startswith("HEAT1D")
+        body += (f'note("shape")\nok(c.raw_call("crom_fom_step", c.CROM_FOM_{kind}, {nb}, {n}, {n if two_d else 1}, '
+                 f"p, p, p, 1e-9, {steps}, p, p + (1 << 34), S))\n")
+    parts = "\n".join(trace(body)).split("shape")[1:]
+    for (kind, n, nb, steps, one), part in zip(FOM_ROUTES, parts, strict=True):
+        ks = kernels(part.splitlines())
+        got = len(ks) == 1 and any(k in ks[0] for k in ("fom_field", "fom_tile", "fom_wide", "fom_line"))
+        assert got == one, (kind, n, nb, steps, ks)
+        assert got or len(ks) == steps, (kind, n, nb, steps, ks)
