@@ -248,7 +248,7 @@ __device__ __forceinline__ int ticket(int* counter, int n) {
 //
 // kAhead: partial rows read ahead of their addition (20 hide the memory latency of a chain
 // of a few hundred samples; the general kernel's 64 registers hold 4).
-template <int kAhead>
+template <int kAhead, bool kPoints = false>
 __device__ __forceinline__ void finish_cta(const FwdParams& p, const float* outv, int ss, int cs, int inst, int first,
                                            int ns, int ntiles, int total, double* rho, double* Amat, double* jd,
                                            double* red2) {
@@ -281,6 +281,7 @@ __device__ __forceinline__ void finish_cta(const FwdParams& p, const float* outv
     }
     return;
   }
+  if constexpr (kPoints) return;  // decode and reconstruction alone
 
   // ---- step: residual per sample (Step 2 at iteration 0), partial normal equations
   for (int i = tid; i < ns * r; i += NT) jd[i] = (double)outv[i / r * ss + (oq + i % r) * cs];
@@ -408,10 +409,12 @@ __device__ __forceinline__ void finish_cta(const FwdParams& p, const float* outv
 
 #include "simt_tile.cuh"
 
-// kJvp: the tangent-velocity decode, whose directional channel is seeded per
-// instance (kept out of the other instantiation, whose register budget it would
-// change).
-template <bool kJvp>
+// What an instantiation serves: the step, decode and reconstruction, or the
+// tangent-velocity decode, whose directional channel is seeded per instance.  Apart, since
+// each has 64 registers (1024 threads): a decode's products leave out the step's reduction
+// and solve.
+enum Serves { kServesStep, kServesPoints, kServesTangent };
+template <Serves kServes>
 __device__ __forceinline__ void fwd_fp32_body(const FwdParams& p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int W = p.width, S = p.S, C = p.C, LD = p.LD, m = p.m, r = p.r;
@@ -435,7 +438,7 @@ __device__ __forceinline__ void fwd_fp32_body(const FwdParams& p) {
 
   // ---- which samples does this CTA own?
   int inst = 0, first = 0, ns = 0, ntiles = 0, msz = 0;
-  if (p.mode == kModeStep) {
+  if constexpr (kServes == kServesStep) {
     inst = blockIdx.x;
     const int t = blockIdx.y;
     const int o0 = __ldg(&p.off[inst]);
@@ -508,7 +511,7 @@ __device__ __forceinline__ void fwd_fp32_body(const FwdParams& p) {
       const int n2 = (p.second == kSecondPerK) ? m : (p.second == kSecondLap ? 1 : 0);
       for (int k = 0; k < n2; ++k) ch[o + k] = 0.f;
       o += n2;
-      if (kJvp) {
+      if (kServes == kServesTangent) {
         const int code = find_instance(p.off, p.n_inst, first + (s < ns ? s : 0));
         ch[o] = __ldg(&p.jvp_seed[(size_t)code * W + u]);
       } else {
@@ -529,19 +532,39 @@ __device__ __forceinline__ void fwd_fp32_body(const FwdParams& p) {
 #pragma unroll
       for (int i = 0; i < 16; ++i) acc[i] = 0.f;
       const float* hcol = Hin + j0;
-#pragma unroll 4
-      for (int k = ks * kper; k < (ks + 1) * kper; ++k) {
-        const float wk = __ldg(&Wt[(size_t)k * W + u]);
-        const float4* h4 = reinterpret_cast<const float4*>(hcol + k * LD);
-        const float4 a = h4[0], b = h4[1], c = h4[2], d = h4[3];
-        acc[0] = fmaf(wk, a.x, acc[0]);  acc[1] = fmaf(wk, a.y, acc[1]);
-        acc[2] = fmaf(wk, a.z, acc[2]);  acc[3] = fmaf(wk, a.w, acc[3]);
-        acc[4] = fmaf(wk, b.x, acc[4]);  acc[5] = fmaf(wk, b.y, acc[5]);
-        acc[6] = fmaf(wk, b.z, acc[6]);  acc[7] = fmaf(wk, b.w, acc[7]);
-        acc[8] = fmaf(wk, c.x, acc[8]);  acc[9] = fmaf(wk, c.y, acc[9]);
-        acc[10] = fmaf(wk, c.z, acc[10]); acc[11] = fmaf(wk, c.w, acc[11]);
-        acc[12] = fmaf(wk, d.x, acc[12]); acc[13] = fmaf(wk, d.y, acc[13]);
-        acc[14] = fmaf(wk, d.z, acc[14]); acc[15] = fmaf(wk, d.w, acc[15]);
+      // The next kWAhead weights are on their way while the current ones are used (kper is a
+      // multiple of 8; the step's registers hold four).  Left to the compiler's unrolling, the
+      // loads in flight, and the time, changed with the code around this loop: 16137 points
+      // of 36 channels, width 96, 7.9 ms, 7.2 so; a step of 204 x 32 samples, r = 32, width
+      // 160, 7.4 and 6.7 ms.
+      constexpr int kWAhead = kServes == kServesStep ? 4 : 8;
+      const int kbeg = ks * kper, kend = kbeg + kper;
+      float next[kWAhead];
+#pragma unroll
+      for (int i = 0; i < kWAhead; ++i) next[i] = __ldg(&Wt[(size_t)(kbeg + i) * W + u]);
+#pragma unroll 1
+      for (int k0 = kbeg; k0 < kend; k0 += kWAhead) {
+        float wv[kWAhead];
+#pragma unroll
+        for (int i = 0; i < kWAhead; ++i) wv[i] = next[i];
+        if (k0 + kWAhead < kend) {
+#pragma unroll
+          for (int i = 0; i < kWAhead; ++i) next[i] = __ldg(&Wt[(size_t)(k0 + kWAhead + i) * W + u]);
+        }
+#pragma unroll
+        for (int i = 0; i < kWAhead; ++i) {
+          const float wk = wv[i];
+          const float4* h4 = reinterpret_cast<const float4*>(hcol + (k0 + i) * LD);
+          const float4 a = h4[0], b = h4[1], c = h4[2], d = h4[3];
+          acc[0] = fmaf(wk, a.x, acc[0]);  acc[1] = fmaf(wk, a.y, acc[1]);
+          acc[2] = fmaf(wk, a.z, acc[2]);  acc[3] = fmaf(wk, a.w, acc[3]);
+          acc[4] = fmaf(wk, b.x, acc[4]);  acc[5] = fmaf(wk, b.y, acc[5]);
+          acc[6] = fmaf(wk, b.z, acc[6]);  acc[7] = fmaf(wk, b.w, acc[7]);
+          acc[8] = fmaf(wk, c.x, acc[8]);  acc[9] = fmaf(wk, c.y, acc[9]);
+          acc[10] = fmaf(wk, c.z, acc[10]); acc[11] = fmaf(wk, c.w, acc[11]);
+          acc[12] = fmaf(wk, d.x, acc[12]); acc[13] = fmaf(wk, d.y, acc[13]);
+          acc[14] = fmaf(wk, d.z, acc[14]); acc[15] = fmaf(wk, d.w, acc[15]);
+        }
       }
       // add the KS partial sums of unit u: thread (u, ks) finishes 16 / KS of the columns
       float* mine = red + ((size_t)ks * W + u) * 16;
@@ -564,12 +587,12 @@ __device__ __forceinline__ void fwd_fp32_body(const FwdParams& p) {
 
   output_layer(p, p.wout, Hin, LD, NP, outv, 0);
   __syncthreads();
-  finish_cta<4>(p, outv, C, 1, inst, first, ns, ntiles, msz, rho, Amat, qs, reinterpret_cast<double*>(red));
+  finish_cta<4, kServes != kServesStep>(p, outv, C, 1, inst, first, ns, ntiles, msz, rho, Amat, qs, reinterpret_cast<double*>(red));
 }
 
-__global__ void __launch_bounds__(1024) fwd_fp32_kernel(FwdParams p) { fwd_fp32_body<false>(p); }
-// up to 1024 threads per CTA: the bound keeps it within 64 registers
-__global__ void __launch_bounds__(1024) fwd_fp32_jvp_kernel(FwdParams p) { fwd_fp32_body<true>(p); }
+// (up to 1024 threads per CTA: the bound keeps it within 64 registers)
+template <Serves kServes>
+__global__ void __launch_bounds__(1024) fwd_fp32_kernel(FwdParams p) { fwd_fp32_body<kServes>(p); }
 
 size_t fwd_smem_bytes(int W, int S, int C, int m, int r, int* LD_out) {
   const int NP = S * C;
@@ -632,7 +655,10 @@ cudaError_t launch_fwd(FwdParams& p, FwdKernel kind, dim3 grid, cudaStream_t s) 
     return cudaLaunchKernelEx(&cfg, kernel, p);
   }
   const size_t smem = fwd_smem_bytes(W, p.S, p.C, p.m, p.r, &p.LD);
-  return p.jvp_seed ? go(fwd_fp32_jvp_kernel, W * kKSplit, smem) : go(fwd_fp32_kernel, W * kKSplit, smem);
+  const auto kernel = p.mode == kModeStep ? fwd_fp32_kernel<kServesStep>
+                      : p.jvp_seed        ? fwd_fp32_kernel<kServesTangent>
+                                          : fwd_fp32_kernel<kServesPoints>;
+  return go(kernel, W * kKSplit, smem);
 }
 
 // The tile kernel's variant for S samples of C channels, or kFwdGeneral if none fits.
