@@ -536,7 +536,7 @@ __device__ __forceinline__ void fwd_fp32_body(const FwdParams& p) {
       // multiple of 8; the step's registers hold four).  Left to the compiler's unrolling, the
       // loads in flight, and the time, changed with the code around this loop: 16137 points
       // of 36 channels, width 96, 7.9 ms, 7.2 so; a step of 204 x 32 samples, r = 32, width
-      // 160, 7.4 and 6.7 ms.
+      // 160, 7.7 and 7.0 ms.
       constexpr int kWAhead = kServes == kServesStep ? 4 : 8;
       const int kbeg = ks * kper, kend = kbeg + kper;
       float next[kWAhead];
@@ -700,16 +700,21 @@ bool small_fits(int W, int S, int C, int m, int r, int hidden) {
 int pick_samples(int W, int C, int m, int r, int want);
 
 // Which kernel N samples of C channels get (decode, reconstruction and step); all three
-// measured on 550 shapes (widths 32 to 256, 1 to 16 channels, 1 to 10^5 samples), with
-// these lines the choice is within 2 % of the best on average and nowhere more than 5 %
-// slower than the general kernel was alone.
-//  * The tile kernel from three warps per SM on (a warp: 8 units x 8 columns a lane), four
-//    for up to four channels: 0.3 to 0.9 of the general kernel's time above the line, 1.2
-//    to 3.5 times it below (one warp per CTA walks all of K: 1362 values of width 256, 471
-//    us against 181 us).  A lone channel needs four at width 128 and more in proportion to
-//    the width, as its chain over K grows while the general kernel splits it; the step's
-//    bound on N counts every instance at its largest, six, in 1D (few
-//    channels, short uneven instances) ten.
+// measured on 1450 shapes (widths 32 to 256, 1 to 36 channels, 1 to 10^5 samples), 900 of
+// them around the lines: with these the choice is 5 % from the best on average there, and
+// nowhere more than 2 % slower than the general kernel was alone.
+//  * The tile kernel from 3.25 warps per SM on (a warp: 8 units x 8 columns a lane): 0.3 to
+//    0.9 of the general kernel's time above the line, 1.2 to 3.5 times it below (one warp
+//    per CTA walks all of K: 1362 values of width 256, 471 us against 181 us).  With two to
+//    four channels from 4.25, and in proportion to the width above 160, as a CTA's chain over K
+//    grows while the general kernel splits it (3364 points of two channels, width 224: 236
+//    against 164 us).  A lone channel needs four at width 128 and so on in proportion; at
+//    width 32 with SIREN 12 (its sines outweigh the products: 50 x 1158 values 131 against
+//    101 us).  One layer has no products at all: seven (3483 points of nine channels, width
+//    64, 17 against 13 us).  The step's bound on N counts every instance at its largest: six,
+//    in 1D (few channels, short uneven instances) ten, of the channels that its iterations
+//    carry on average (seven instances of 415 samples, r = 1, three iterations: 657 against
+//    591 us).
 //  * Else the latency kernel, two samples per CTA where one would not fit the GPU at once
 //    (200 samples of a 2D step: 67 us with two, 91 us with one per CTA), if its CTAs take
 //    no more rounds of the GPU than (C + 1) / 2 (step: C / 2): its time grows with the rounds, the
@@ -717,11 +722,15 @@ int pick_samples(int W, int C, int m, int r, int want);
 //    channels of 600: 0.9 times).  Width 32 and two layers leave too little to gain in a
 //    second round, three layers in a third.
 //  * Else the general kernel.
-bool tile_pays(const crom_ctx* ctx, long long N, int C, bool step) {
+bool tile_pays(const crom_ctx* ctx, long long columns, int C, bool step) {  // columns: N C
   const int W = ctx->desc.width;
-  const long long warps = N * C * W / 2048, sms = ctx->num_sms;
-  if (step) return warps >= (ctx->desc.m == 1 ? 10 : 6) * sms;
-  return C > 1 ? warps >= (C > 4 ? 3 : 4) * sms : warps >= std::max(3 * sms, 4 * sms * W / 128);
+  const long long warps = columns * W / 2048, sms = ctx->num_sms;
+  long long quarters;  // of a warp per SM
+  if (step) quarters = ctx->desc.m == 1 ? 40 : 24;
+  else if (ctx->desc.hidden == 1) quarters = 28;
+  else if (C == 1) quarters = W == 32 && ctx->desc.activation == CROM_ACT_SIREN ? 48 : std::max(12, W / 8);
+  else quarters = C > 4 ? 13 : std::max(17, W / 8 - 4);
+  return 4 * warps >= quarters * sms;
 }
 bool small_pays(const crom_ctx* ctx, long long N, int S, int C, bool step) {
   const long long ctas = (N + S - 1) / S, rounds = (ctas + ctx->num_sms - 1) / ctx->num_sms;
@@ -732,7 +741,7 @@ bool small_pays(const crom_ctx* ctx, long long N, int S, int C, bool step) {
 FwdKernel plan_points(const crom_ctx* ctx, long long sets, long long n, int C, int general_want, int* S) {
   const int W = ctx->desc.width, m = ctx->desc.m, r = ctx->desc.r;
   const long long N = sets * n;
-  if (tile_pays(ctx, N, C, false)) {
+  if (tile_pays(ctx, N * C, C, false)) {
     const FwdKernel k = tile_plan(ctx, sets, n, C, S);
     if (k != kFwdGeneral) return k;
   }
@@ -866,12 +875,13 @@ int step_samples_per_cta(const crom_ctx* ctx, int n_inst, int max_samples) {
 
 // Kernel, samples per CTA (S) and per partial row (PS, which bounds the grid and the
 // scratch, and fixes the order of the FP64 sums) of the FP32 step.
-FwdKernel plan_step(const crom_ctx* ctx, int n_inst, int max_samples, int* S, int* PS) {
+FwdKernel plan_step(const crom_ctx* ctx, int n_inst, int max_samples, int gn_iters, int* S, int* PS) {
   const int W = ctx->desc.width, m = ctx->desc.m, r = ctx->desc.r;
   const int C0 = ChannelSet{m, kSecondLap, r}.count(m);
   *PS = step_samples_per_cta(ctx, n_inst, max_samples);
   const long long N = (long long)n_inst * max_samples;
-  if (tile_pays(ctx, N, C0, true)) {
+  const int gn = gn_iters, C = C0 + (gn - 1) * (r + 2);  // later iterations carry r + 2 channels
+  if (tile_pays(ctx, N * C / gn, C0, true)) {
     const FwdKernel k = tile_plan(ctx, n_inst, max_samples, C0, S);
     if (k != kFwdGeneral) return k;
   }
@@ -896,7 +906,7 @@ cudaError_t launch_step_fp32(crom_ctx* ctx, const crom_step_desc* step, int n_in
   fill_decoder(p, ctx);
   const int m = p.m, r = p.r;
   int S, PS;
-  const FwdKernel kind = plan_step(ctx, n_inst, max_samples, &S, &PS);
+  const FwdKernel kind = plan_step(ctx, n_inst, max_samples, step->gn_iters, &S, &PS);
   const int max_tiles = (max_samples + PS - 1) / PS;  // partial rows per instance
   const int n_entries = r * (r + 1) / 2 + r;
 
@@ -1014,7 +1024,7 @@ cudaError_t launch_step_fp32_noalloc(const crom_ctx* ctx, const crom_step_desc* 
   fill_decoder(p, ctx);
   const int m = p.m, r = p.r;
   int S, PS;
-  const FwdKernel kind = plan_step(ctx, n_inst, max_samples, &S, &PS);
+  const FwdKernel kind = plan_step(ctx, n_inst, max_samples, step->gn_iters, &S, &PS);
   const int max_tiles = (max_samples + PS - 1) / PS;  // partial rows per instance
   const int n_entries = r * (r + 1) / 2 + r;
   // layout inside the static array

@@ -219,3 +219,35 @@ def test_full_order_steps_take_the_faster_launches(trace):
         got = len(ks) == 1 and any(k in ks[0] for k in ("fom_field", "fom_tile", "fom_wide", "fom_line"))
         assert got == one, (kind, n, nb, steps, ks)
         assert got or len(ks) == steps, (kind, n, nb, steps, ks)
+
+
+# m, r, width, layers, activation, call, points (or codes x points), the kernel: shapes at
+# which the tile kernel was measured slower than the general one, and above the lines
+FP32_ROUTES = [(3, 1, 224, 4, 0, "decode 17", 3364, "fwd_fp32"), (3, 1, 224, 4, 0, "decode 17", 4200, "fwd_tile"),
+               (2, 2, 128, 3, 0, "decode 16", 3264, "fwd_fp32"), (2, 2, 128, 3, 0, "decode 16", 3800, "fwd_tile"),
+               (1, 12, 224, 5, 0, "tangent", 3492, "fwd_fp32"), (1, 12, 224, 5, 0, "tangent", 4500, "fwd_tile"),
+               (2, 1, 32, 5, 1, "recon 42", 926, "fwd_fp32"), (2, 1, 32, 5, 1, "recon 42", 3000, "fwd_tile"),
+               (2, 1, 32, 5, 0, "recon 42", 926, "fwd_tile"), (3, 4, 64, 1, 0, "decode 27", 3483, "fwd_fp32"),
+               (3, 4, 64, 1, 0, "decode 27", 4500, "fwd_tile"), (2, 8, 128, 5, 0, "decode 31", 16384, "fwd_tile"),
+               (2, 16, 256, 5, 0, "recon 8", 65536, "fwd_tile")]
+
+
+def test_fp32_calls_take_the_faster_kernel(trace):
+    body = "p = 0x7f0000000000          # not read: no kernel runs\n"
+    for m, r, W, L, act, call, n, _ in FP32_ROUTES:
+        name, arg = (call + " 0").split()[:2]
+        body += f"""h, d = ctypes.c_void_p(), c.crom_decoder_desc({m}, {r}, {W}, {L}, {act}, 5.0)
+ok(c.raw_call("crom_create", ctypes.byref(h), ctypes.byref(d), 0))
+w = np.ascontiguousarray(gen.pack_params(gen.xavier_decoder(gen.DecoderSpec({m}, {r}, {W}, {L}), seed=1)), np.float32)
+ok(c.raw_call("crom_set_weights", h, w.ctypes.data, w.size, 0, S))
+note("shape")
+if "{name}" == "decode":
+    ok(c.raw_call("crom_decode", h, 1, p, p, p, {n}, {arg}, p, S))
+elif "{name}" == "tangent":
+    ok(c.raw_call("crom_tangent_velocity", h, 1, p, p, 1e-3, p, p, {n}, p, S))
+else:
+    ok(c.raw_call("crom_reconstruct", h, c.CROM_PREC_FP32, {arg}, p, {n}, p, p, S))
+"""
+    parts = "\n".join(trace(body)).split("shape")[1:]
+    for shape, part in zip(FP32_ROUTES, parts, strict=True):
+        assert shape[-1] in kernels(part.splitlines())[-1], shape
