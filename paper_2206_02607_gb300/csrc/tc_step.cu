@@ -1244,15 +1244,27 @@ namespace {
 // groups for a second round of equal ones.  Measured, two iterations, F16X2, whole against
 // split: 1 x 200 samples 342 / 67 us, 8 x 4096 8899 / 240 us, 450 x (32..512) 1140 / 603 us,
 // 700 x 256 1084 / 785 us; but 608 x 256 611 / 637 us and 1024 x (32..512) 1156 / 1213 us.
-// Far above one instance per group only the caller's bound on |M_i| could ask for it.
-bool split_wanted(int n_inst, int n_samples, int max_samples, int tile, int num_sms) {
+// Far above one instance per group only the caller's bound on |M_i| could ask for it.  With
+// more tiles than groups the iterations also pay their launches and uneven ends: near one
+// instance per group, and from the second iteration on with two layers (whose tiles are
+// short: three in F16X2, two in F16), more has to be gained (244 x 96 samples, two layers,
+// F16, 160 against 195 us; 597 instances of 17043 in all, F16X2, 137 against 162 us).  Of
+// 800 shapes around these lines one, dealt, is more than 1 % slower (82 against 89 us).
+bool split_wanted(int n_inst, int n_samples, int max_samples, int tile, int num_sms, int hidden, int gn_iters, bool lo_parts) {
   const double G = kGroups * num_sms;
-  // (the prefix sums of the tiles are 32-bit, whatever the offsets)
-  if (n_inst > 1.25 * G || ceil((double)std::min(max_samples, n_samples) / tile) * n_inst >= 2147483648.0) return false;
-  const double mean = (double)n_samples / n_inst / tile, T = (mean + 0.5) * n_inst;
   const double largest = ceil((double)std::min(max_samples, n_samples) / tile);
+  // (the prefix sums of the tiles are 32-bit, whatever the offsets)
+  if (n_inst > 1.25 * G || largest * n_inst >= 2147483648.0) return false;
+  const double mean = (double)n_samples / n_inst / tile;
+  const bool even = (double)max_samples * n_inst <= 1.05 * n_samples;
+  const double T = even ? largest * n_inst : (mean + 0.5) * n_inst;
   const double whole = largest <= 1.25 * mean ? std::max(largest, ceil(n_inst / G) * mean) : largest;
-  return whole >= ceil(T / G) + 1.0 && whole >= 1.15 * T / G;
+  double gain = 1.0;  // in tiles per group
+  if (T > G) {
+    if (n_inst > 0.87 * G) gain = gn_iters == 1 ? 2.0 : 2.5;
+    if (hidden == 2 && gn_iters > 1) gain = std::max(gain, lo_parts ? 3.0 : 2.0);
+  }
+  return whole >= ceil(T / G) + gain && whole >= 1.15 * T / G;
 }
 }  // namespace
 
@@ -1283,7 +1295,8 @@ cudaError_t launch_step_tc(crom_ctx* ctx, const crom_step_desc* step, int lo_par
   // Split mode: see split_wanted.  Its tile rows are sized for every instance's ragged
   // last tile; without them the groups take whole instances, which gives the same bits.
   const int tile = lo_parts ? kLarge : 2 * kLarge, n_entries = ctx->desc.r * (ctx->desc.r + 3) / 2;
-  bool split = step->line_search == 0 && !small_tiles && split_wanted(n_inst, n_samples, max_samples, tile, ctx->num_sms);
+  bool split = step->line_search == 0 && !small_tiles && split_wanted(n_inst, n_samples, max_samples, tile, ctx->num_sms,
+                                                                           ctx->desc.hidden, step->gn_iters, lo_parts != 0);
   const int tile_rows = n_samples / tile + n_inst, deal_grid = std::min(tile_rows, ctx->num_sms);
   if (split)
     e = try_grow_kept(ctx, s, &ctx->deal_rows, &ctx->deal_rows_cap,

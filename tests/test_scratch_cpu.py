@@ -251,3 +251,21 @@ else:
     parts = "\n".join(trace(body)).split("shape")[1:]
     for shape, part in zip(FP32_ROUTES, parts, strict=True):
         assert shape[-1] in kernels(part.splitlines())[-1], shape
+
+
+# layers, sizes, precision, iterations, whether the tiles are dealt: shapes at which the
+# dealt form was measured slower than whole instances (False), and their neighbours
+DEAL_ROUTES = [(2, "[96] * 244", "F16", 2, False), (5, "[96] * 244", "F16", 2, True), (2, "[96] * 200", "F16", 2, True),
+               (2, "[32] * 627", "F16X2", 3, False), (5, "[73] * 430", "F16", 3, False), (5, "[140] * 430", "F16", 3, True),
+               (3, "[20, 54] * 298", "F16X2", 2, False), (5, "[4096] * 8", "F16", 2, True), (2, "[200]", "F16X2", 2, True)]
+
+
+def test_tiles_are_dealt_where_that_is_faster(trace):
+    body = ""
+    for hidden, sizes, prec, gn, _ in DEAL_ROUTES:
+        body += f'h = context(hidden={hidden})\nnote("shape")\nstep(h, {sizes}, c.CROM_PREC_{prec}, gn={gn})\n'
+    parts = "\n".join(trace(body)).split("shape")[1:]
+    for (hidden, sizes, prec, gn, dealt), part in zip(DEAL_ROUTES, parts, strict=True):
+        ks = kernels(part.splitlines())
+        assert (not any("order" in k for k in ks)) == dealt, (hidden, sizes, prec, gn, ks)
+        assert len(ks) == (gn if dealt else 2), ks
