@@ -12,7 +12,7 @@ namespace crom {
 // Warp-parallel FP64 Cholesky solve of A x = b, r <= 32, with A = a[i*(r+1)+j] in
 // shared memory (both triangles) and b in column r.  Status: NONFINITE when A or b holds
 // a NaN/Inf, SINGULAR when a pivot is <= 1e-14 * max diag(A); on success x_k is left in
-// a[k*(r+1)+r].  invd: r doubles of shared scratch.  All 32 lanes of the warp must call it.
+// a[k*(r+1)+r].  All 32 lanes of the warp must call it.
 //
 // A single warp's FP64 instruction takes 64 clocks here whatever its active lanes, and a
 // reciprocal square root about 380, so the chain is kept short: right-looking, the
@@ -21,7 +21,7 @@ namespace crom {
 // r = 8, not the longest row's length), the back substitution in registers.  Every entry
 // sees the same operations in the same order as the row-per-lane form (17k clocks at
 // r = 8, this form 9.7k).
-__device__ __forceinline__ int chol_solve_warp(double* A, double* invd, int r, int lane) {
+__device__ __forceinline__ int chol_solve_warp(double* A, int r, int lane) {
   const int R = r + 1;
   // FP64 comparisons and conversions cost as much as additions: the checks compare bit
   // patterns (non-negative doubles order like integers)

@@ -394,8 +394,7 @@ __device__ __forceinline__ void finish_cta(const FwdParams& p, const float* outv
   __syncthreads();
   if (tid < 32) {
     // Cholesky A = L L^T and the two triangular solves, spread over one warp
-    __shared__ double s_invd[kMaxR];
-    const int st = chol_solve_warp(Amat, s_invd, r, tid);
+    const int st = chol_solve_warp(Amat, r, tid);
     if (st == CROM_OK && tid < r) {
       if (p.iter == 0) p.qbase[(size_t)inst * r + tid] = p.qio[(size_t)inst * r + tid];
       p.qio[(size_t)inst * r + tid] += Amat[tid * (r + 1) + r];

@@ -155,7 +155,6 @@ struct __align__(16) Group {
   double delta[16];   // line search: the GN direction
   double phi0, phi, slope;
   double amat[15 * 16];
-  double invd[16];
   float c1[kTcWidth];
   float dz1[kTcWidth];
   float dmax[4];
@@ -963,7 +962,7 @@ __device__ __forceinline__ bool run_iteration(Lane& c, const StepParams& p, Own&
       if (c.gw == 0) {
         int st = CROM_ERR_TIMEOUT;
         if (last == 1) {
-          st = chol_solve_warp(G->amat, G->invd, r, c.gt);
+          st = chol_solve_warp(G->amat, r, c.gt);
           if (st == CROM_OK && c.gt < r) {
             if (kMode == kIterFirst) p.qbase[(size_t)inst * r + c.gt] = G->qn[c.gt];
             p.q[(size_t)inst * r + c.gt] = G->qcur[c.gt] + G->amat[c.gt * R + r];
@@ -1131,7 +1130,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_tc_kernel(StepParams p) {
       group_sync(c.g);
       if (c.gw == 0) {
         const double minus_v = c.gt < r ? G->amat[c.gt * R + r] : 0.0;  // -(J^T rho)_k
-        const int st = chol_solve_warp(G->amat, G->invd, r, c.gt);
+        const int st = chol_solve_warp(G->amat, r, c.gt);
         if (st == CROM_OK && c.gt < r) {
           const double d = G->amat[c.gt * R + r];
           if (p.line_search > 0) G->delta[c.gt] = d;
