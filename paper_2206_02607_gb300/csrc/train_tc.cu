@@ -381,7 +381,7 @@ cudaError_t trainer_tc_alloc(crom_trainer* t) {
   c.colpart = (float*)A((size_t)L * tiles_m * 4 * w * 4);
   c.rowpart = (float*)A((size_t)tiles_m * 4 * 2 * 4);
   c.colmid = (float*)A((size_t)L * ((tiles_m * 4 + kColPer - 1) / kColPer) * w * 4);
-  c.split = (float*)A((size_t)(L - 1) * kSplitsW * w * w * 4);
+  c.split = (float*)A((size_t)(L - 1) * tc_gemm_splits_used((int)N, kSplitsW) * w * w * 4);
   const int m = t->dec.m;
   c.xin = (float*)A((size_t)N * m * 4);
   c.c0 = (float*)A((size_t)t->B * w * 4);
@@ -402,7 +402,8 @@ cudaError_t trainer_decoder_tc(crom_trainer* t, double* loss_out, int num_sms, c
   const long N = (long)t->B * t->S;
   const int tiles_m = (int)((N + 127) / 128);
   const int parts = tiles_m * 4;
-  const long set = (long)parts * w, split = (long)kSplitsW * w * w;
+  const int splits = tc_gemm_splits_used((int)N, kSplitsW);
+  const long set = (long)parts * w, split = (long)splits * w * w;
   auto& c = t->tc;
   const TrainerLayout& lay = t->lay;
   const float* p = t->params;
@@ -494,7 +495,7 @@ cudaError_t trainer_decoder_tc(crom_trainer* t, double* loss_out, int num_sms, c
   for (int h = 1; h < L; ++h) {
     sums.part[L - 1 + h] = c.split + (h - 1) * split;
     sums.out[L - 1 + h] = gr + lay.dec_w[h];
-    sums.nparts[L - 1 + h] = tc_gemm_splits_used((int)N, kSplitsW);
+    sums.nparts[L - 1 + h] = splits;
     sums.n[L - 1 + h] = (long)w * w;
   }
   sums_level2_kernel<<<dim3(nblk((long)w * w, 128), 2 * L - 1), 128, 0, s>>>(sums);

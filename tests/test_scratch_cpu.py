@@ -192,6 +192,23 @@ def test_a_recorded_step_within_earlier_sizes_allocates_nothing(trace, warm, cal
     assert len(kernels(part)) == 2 and ("order" in kernels(part)[0]) == whole
 
 
+@pytest.mark.parametrize("B,S", [(2, 64), (1, 4000), (64, 4096)])
+def test_mixed_precision_buffers_are_of_the_stated_size(trace, B, S):
+    """The sizes that crom_trainer_set_precision states: two bytes per point, unit and
+    activation array, and a weight gradient's partial sums for the K ranges in use.  A tenth
+    more and a megabyte for the column sums and the small arrays."""
+    w, L = 256, 5
+    lines = trace(f"""
+        t, d = ctypes.c_void_p(), c.crom_decoder_desc(2, 8, {w}, {L})
+        ok(c.raw_call("crom_trainer_create", ctypes.byref(t), ctypes.byref(d), 4096, {B}, {S}, 0))
+        note("mixed")
+        ok(c.raw_call("crom_trainer_set_precision", t, c.CROM_PREC_BF16_MIXED))
+    """)
+    made = sum(int(x.split()[2]) for x in lines[lines.index("mixed"):] if x.startswith("malloc #"))
+    stated = (L + 2) * B * S * w * 2 + (L - 1) * min(64, -(-B * S // 64)) * w * w * 4
+    assert stated / 2 < made < 1.1 * stated + (1 << 20), (made, stated)
+
+
 # kind, side, ny, fields, steps, whether the steps are one launch: shapes at which the one
 # launch was measured slower than a launch per step (False), and their neighbours
 FOM_ROUTES = [("HEAT2D_NEUMANN_FIELD", 127, 10, 4, False), ("HEAT2D_NEUMANN_FIELD", 127, 10, 50, True),
