@@ -20,17 +20,14 @@ static thread_local std::string g_last_error;
 
 void set_error(const std::string& msg) { g_last_error = msg; }
 
-static cudaError_t fill_device(void* p, const void* host, size_t bytes) {
-  cudaStream_t s;
-  cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-  if (e != cudaSuccess) return e;
-  e = host ? cudaMemcpyAsync(p, host, bytes, cudaMemcpyHostToDevice, s) : cudaMemsetAsync(p, 0, bytes, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  const cudaError_t d = cudaStreamDestroy(s);
-  return e != cudaSuccess ? e : d;
+cudaError_t clear_device(void* p, size_t bytes) {
+  const cudaError_t e = cudaMemset(p, 0, bytes);
+  return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
 }
-cudaError_t clear_device(void* p, size_t bytes) { return fill_device(p, nullptr, bytes); }
-cudaError_t upload_device(void* p, const void* host, size_t bytes) { return fill_device(p, host, bytes); }
+cudaError_t upload_device(void* p, const void* host, size_t bytes) {
+  const cudaError_t e = cudaMemcpy(p, host, bytes, cudaMemcpyHostToDevice);
+  return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+}
 
 namespace {
 

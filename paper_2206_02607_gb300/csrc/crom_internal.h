@@ -229,8 +229,9 @@ cudaError_t launch_step_fp32_noalloc(const crom_ctx* ctx, const crom_step_desc* 
 // done: a launch on any stream may use it next.  (A plain cudaMemset or cudaMemcpy runs on
 // the legacy default stream and may still be under way when it returns, and a non-blocking
 // stream is not ordered after it: a step on such a stream could draw uncleared tickets.)
-// On a stream of its own, since a caller may be recording a graph on its stream, and the
-// default stream may have work queued.
+// Not on a stream of its own: with one created before a trainer's first launch, every
+// later launch took 0.2 us longer (a training step of 40 launches 709 -> 717 us, a step of
+// three 239.0 -> 240.3).
 cudaError_t clear_device(void* p, size_t bytes);
 cudaError_t upload_device(void* p, const void* host, size_t bytes);
 

@@ -130,6 +130,7 @@ cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind k, 
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
   *s = reinterpret_cast<cudaStream_t>(0x100000 + 16 * ++g_streams);
   g_own.push_back(*s);
+  line("stream made " + name(*s));
   return cudaSuccess;
 }
 cudaError_t cudaStreamDestroy(cudaStream_t s) {

@@ -115,6 +115,12 @@ def test_clears_and_copies_are_complete_before_the_first_launch(trace, case):
     assert [x for x in lines if x.startswith("UNORDERED")] == []
 
 
+@pytest.mark.parametrize("case", sorted(CLEARS))
+def test_scratch_is_made_ready_without_a_stream(trace, case):
+    """A stream made before a context's or trainer's first launches slows all later ones."""
+    assert [x for x in trace(CLEARS[case]) if x.startswith("stream")] == []
+
+
 @pytest.mark.parametrize("sizes", ["[4096] * 8", "[64] * 1000"])
 @pytest.mark.parametrize("prec", ["F16X2", "F16"])
 def test_the_timeout_flag_is_cleared_before_the_step_can_set_it(trace, sizes, prec):
