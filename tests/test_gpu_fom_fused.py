@@ -78,3 +78,11 @@ def test_1d_one_launch(c, P):
             for _ in range(steps):
                 ref = O.fom_heat1d_step(ref, dt, coef[b].astype(np.float64))
             assert rel_l2(got[b], ref) < 4 * steps * 2.0 ** -24
+
+
+# more fields than the GPU holds at once, of sides without a wide kernel: clusters of two
+# to eight CTAs, and one CTA per field with two of them on an SM
+@pytest.mark.parametrize("model", ["heat", "heat_field", "upwind", "central"])
+@pytest.mark.parametrize("n,nb", [(57, 400), (96, 700), (164, 400), (200, 300), (252, 310)])
+def test_2d_one_launch_of_many_fields(c, model, n, nb):
+    test_2d_one_launch(c, model, n, nb)
