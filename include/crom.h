@@ -242,9 +242,14 @@ int crom_device_flags(crom_ctx* ctx, int* flags, crom_stream stream);
  *   instance over several CTAs (the last CTA to finish reduces and solves); the
  *   context grows its scratch on first use, so the first call for a given size
  *   must not be made during stream capture.
- * precision CROM_PREC_F16X2 or CROM_PREC_F16: one persistent launch per step
- *   (plus a small ordering kernel); each of a CTA's four 128-thread groups takes
- *   whole instances, largest |M_i| first, from a queue. */
+ * precision CROM_PREC_F16X2 or CROM_PREC_F16: for batches that fill the GPU one
+ *   persistent launch per step (plus a small ordering kernel); each of a CTA's four
+ *   128-thread groups takes whole instances, largest |M_i| first, from a queue.  Few or
+ *   uneven instances take one launch per GN iteration, their sample tiles dealt to all
+ *   groups (the same bits); with line search, in a context tuned to 8-sample tiles
+ *   (crom_autotune), where the tile rows' scratch cannot be had, and in a recorded step
+ *   whose scratch is not there yet, a group keeps its whole instance.  Scratch grows on
+ *   first use, as above. */
 int crom_step(crom_ctx* ctx, const crom_step_desc* step, int precision, int n_inst, double* q,
               const float* alpha, const float* vel, const int* s_off, const float* samples,
               int n_samples, int max_samples, int* status, crom_stream stream);

@@ -10,10 +10,10 @@
 //    Bound by the FP32 pipe for many fields (17 operations a node for advection,
 //    6 for heat, where the step-by-step kernels move 16 and 8 bytes a node through HBM
 //    or L2), by the barrier's latency for few.
-//    8 fields of 128^2, heat, 100 steps: 409 -> 51 us.
+//    8 fields of 128^2, heat, 100 steps: 410 -> 53 us; 400 of 200^2, 20 steps: 1230 -> 408.
 //  * fom_wide_kernel: the same for many fields of sides 128 and 256.  64 fields of 256^2,
-//    advection-diffusion, 10 steps: 96 -> 47 us (512 fields: 781 -> 379; 1024 fields of
-//    128^2, heat: 202 -> 60).
+//    advection-diffusion, 10 steps: 84 -> 48 us with the velocities in L2 from the call
+//    before (96 -> 54 without; 512 fields: 784 -> 379; 1024 fields of 128^2, heat: 203 -> 60).
 //  * fom_line_kernel (1D) and fom_field_kernel (2D, other sides up to kFieldMaxHeat and
 //    kFieldMaxAdv): one CTA per field, the field twice in shared memory, one barrier per
 //    step (100 steps of 256 nodes: 409 -> 14 us; 10 steps of 97^2, heat: 41 -> 24 us).
@@ -218,7 +218,12 @@ inline int tile_thr(int n, int RT, int NC) { return (n / 4 * ((n / RT + NC - 1) 
 
 // The same for many fields of sides 128 and 256: 1024 threads per CTA (64 registers), so
 // that a field takes a quarter of the CTAs and clusters of four pack onto the GPU (of the
-// eight-CTA clusters about twelve run at a time: 64 fields of 256^2 took 70 us).  The
+// eight-CTA clusters about twelve run at a time: 64 fields of 256^2 took 70 us).  Those two
+// sides alone: a row is then one or two whole warps, which the lane exchange needs, and
+// the CTA's 1024 threads divide into rows.  Other sides stay with fom_tile_kernel, 0.32 to
+// 0.59 of a launch per step's time where the GPU is full (400 fields of 200^2, five steps:
+// heat 138 against 329 us, advection 192 against 388; 300 of 252^2, ten: 213 against 676
+// and 292 against 800; 800 of 180^2, upwind, ten: 663 against 1127).  The
 // face velocities (or the coefficient field) lie in shared memory; column neighbours and
 // the fluxes through the tiles' sides come from the adjacent lanes, what crosses the two
 // warps of a 256-node row and the rows at the tiles' borders through shared memory.
