@@ -717,7 +717,15 @@ int pick_samples(int W, int C, int m, int r, int want);
 //    64, 17 against 13 us).  The step's bound on N counts every instance at its largest: six,
 //    in 1D (few channels, short uneven instances) ten, of the channels that its iterations
 //    carry on average (seven instances of 415 samples, r = 1, three iterations: 657 against
-//    591 us).
+//    591 us).  A bound far above the samples that there are gives CTAs without work: of
+//    these four (one instance of 1768 samples bounded by 6284, width 32: 364 against 251 us),
+//    20 for more than ten channels of width 32 (95 instances, r = 6, four layers: 435
+//    against 397).  One layer has only the channels' activations to gain from: ten (in 1D
+//    15), and a width of seven times the channels (two instances of 2181 samples, r = 8,
+//    width 64: 185 against 131 us).  Both take at least 64 and four instances: the small
+//    CTAs' threads are alone with a long instance's sums (two of 20000 samples, 13 channels,
+//    width 32: 1961 against 1666 us).  By 1300 steps, half of them of one layer: two above
+//    1.015 of the general kernel's time (1.042, 1.017), 0.66 on average where tiles are used.
 //  * Else the latency kernel, two samples per CTA where one would not fit the GPU at once
 //    (200 samples of a 2D step: 67 us with two, 91 us with one per CTA), if its CTAs take
 //    no more rounds of the GPU than (C + 1) / 2 (step: C / 2): its time grows with the rounds, the
@@ -725,12 +733,18 @@ int pick_samples(int W, int C, int m, int r, int want);
 //    channels of 600: 0.9 times).  Width 32 and two layers leave too little to gain in a
 //    second round, three layers in a third.
 //  * Else the general kernel.
-bool tile_pays(const crom_ctx* ctx, long long columns, int C, bool step) {  // columns: N C
+// (columns: N C; held: a step's, of the samples that there are)
+bool tile_pays(const crom_ctx* ctx, long long columns, int C, bool step, long long held = 0, int n_inst = 0) {
   const int W = ctx->desc.width;
   const long long warps = columns * W / 2048, sms = ctx->num_sms;
   long long quarters;  // of a warp per SM
-  if (step) quarters = ctx->desc.m == 1 ? 40 : 24;
-  else if (ctx->desc.hidden == 1) quarters = 28;
+  if (step) {
+    const bool one = ctx->desc.hidden == 1;
+    const bool narrow = W == 32 && C > 10;
+    const int least = one ? (ctx->desc.m == 1 ? 15 : 10) : narrow ? 20 : 4;
+    if ((one && (7 * C > W || n_inst < 4)) || (!one && narrow && n_inst < 64) || held * W / 2048 < least * sms) return false;
+    quarters = ctx->desc.m == 1 ? 40 : 24;
+  } else if (ctx->desc.hidden == 1) quarters = 28;
   else if (C == 1) quarters = W == 32 && ctx->desc.activation == CROM_ACT_SIREN ? 48 : std::max(12, W / 8);
   else quarters = C > 4 ? 13 : std::max(17, W / 8 - 4);
   return 4 * warps >= quarters * sms;
@@ -878,13 +892,13 @@ int step_samples_per_cta(const crom_ctx* ctx, int n_inst, int max_samples) {
 
 // Kernel, samples per CTA (S) and per partial row (PS, which bounds the grid and the
 // scratch, and fixes the order of the FP64 sums) of the FP32 step.
-FwdKernel plan_step(const crom_ctx* ctx, int n_inst, int max_samples, int gn_iters, int* S, int* PS) {
+FwdKernel plan_step(const crom_ctx* ctx, int n_inst, int n_samples, int max_samples, int gn_iters, int* S, int* PS) {
   const int W = ctx->desc.width, m = ctx->desc.m, r = ctx->desc.r;
   const int C0 = ChannelSet{m, kSecondLap, r}.count(m);
   *PS = step_samples_per_cta(ctx, n_inst, max_samples);
   const long long N = (long long)n_inst * max_samples;
   const int gn = gn_iters, C = C0 + (gn - 1) * (r + 2);  // later iterations carry r + 2 channels
-  if (tile_pays(ctx, N * C / gn, C0, true)) {
+  if (tile_pays(ctx, N * C / gn, C0, true, std::min<long long>(N, n_samples) * C / gn, n_inst)) {
     const FwdKernel k = tile_plan(ctx, n_inst, max_samples, C0, S);
     if (k != kFwdGeneral) return k;
   }
@@ -909,7 +923,7 @@ cudaError_t launch_step_fp32(crom_ctx* ctx, const crom_step_desc* step, int n_in
   fill_decoder(p, ctx);
   const int m = p.m, r = p.r;
   int S, PS;
-  const FwdKernel kind = plan_step(ctx, n_inst, max_samples, step->gn_iters, &S, &PS);
+  const FwdKernel kind = plan_step(ctx, n_inst, n_samples, max_samples, step->gn_iters, &S, &PS);
   const int max_tiles = (max_samples + PS - 1) / PS;  // partial rows per instance
   const int n_entries = r * (r + 1) / 2 + r;
 
@@ -1027,7 +1041,7 @@ cudaError_t launch_step_fp32_noalloc(const crom_ctx* ctx, const crom_step_desc* 
   fill_decoder(p, ctx);
   const int m = p.m, r = p.r;
   int S, PS;
-  const FwdKernel kind = plan_step(ctx, n_inst, max_samples, step->gn_iters, &S, &PS);
+  const FwdKernel kind = plan_step(ctx, n_inst, n_samples, max_samples, step->gn_iters, &S, &PS);
   const int max_tiles = (max_samples + PS - 1) / PS;  // partial rows per instance
   const int n_entries = r * (r + 1) / 2 + r;
   // layout inside the static array

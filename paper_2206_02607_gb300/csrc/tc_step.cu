@@ -1249,6 +1249,10 @@ namespace {
 // short: three in F16X2, two in F16), more has to be gained (244 x 96 samples, two layers,
 // F16, 160 against 195 us; 597 instances of 17043 in all, F16X2, 137 against 162 us).  Of
 // 800 shapes around these lines one, dealt, is more than 1 % slower (82 against 89 us).
+// Instances of a tile or less on average may all be of one tile, whatever their bound: they
+// stay whole unless it is five tiles (20 instances of 15 samples bounded by 60, F16X2, three
+// iterations: 74 against 97 us; with one of 60 it would be 100).  Two tiles of F16X2 are no
+// faster dealt from the second iteration on (one instance of 22, r = 15: 111 against 119 us).
 bool split_wanted(int n_inst, int n_samples, int max_samples, int tile, int num_sms, int hidden, int gn_iters, bool lo_parts) {
   const double G = kGroups * num_sms;
   const double largest = ceil((double)std::min(max_samples, n_samples) / tile);
@@ -1258,7 +1262,8 @@ bool split_wanted(int n_inst, int n_samples, int max_samples, int tile, int num_
   const bool even = (double)max_samples * n_inst <= 1.05 * n_samples;
   const double T = even ? largest * n_inst : (mean + 0.5) * n_inst;
   const double whole = largest <= 1.25 * mean ? std::max(largest, ceil(n_inst / G) * mean) : largest;
-  double gain = 1.0;  // in tiles per group
+  if (mean <= 1.0 && largest < 5.0) return false;
+  double gain = T <= G && lo_parts && gn_iters > 1 ? 2.0 : 1.0;  // in tiles per group
   if (T > G) {
     if (n_inst > 0.87 * G) gain = gn_iters == 1 ? 2.0 : 2.5;
     if (hidden == 2 && gn_iters > 1) gain = std::max(gain, lo_parts ? 3.0 : 2.0);

@@ -35,12 +35,12 @@ PRELUDE = """
         keep.append(p)
         ok(c.raw_call("crom_set_weights", h, p.ctypes.data, p.size, 0, S))
         return h
-    def step(h, sizes, prec, gn=2, r=8, m=2, stream=S, status=0):
+    def step(h, sizes, prec, gn=2, r=8, m=2, stream=S, status=0, bound=0):
         n, tot = len(sizes), int(sum(sizes))
         sd = c.crom_step_desc(c.CROM_PDE_HEAT, gn, 1e-5)
         rc = c.raw_call("crom_step", h, ctypes.byref(sd), prec, n, arr(np.zeros((n, r)), np.float64),
                         arr(np.ones(n), np.float32), None, arr(gen.ragged_offsets(np.array(sizes)), np.int32),
-                        arr(np.zeros((tot, m)), np.float32), tot, max(sizes), arr(np.zeros(n), np.int32), stream)
+                        arr(np.zeros((tot, m)), np.float32), tot, bound or max(sizes), arr(np.zeros(n), np.int32), stream)
         assert rc == status, (rc, c.last_error())
 """ % ROOT
 
@@ -292,3 +292,37 @@ def test_tiles_are_dealt_where_that_is_faster(trace):
         ks = kernels(part.splitlines())
         assert (not any("order" in k for k in ks)) == dealt, (hidden, sizes, prec, gn, ks)
         assert len(ks) == (gn if dealt else 2), ks
+
+
+# layers, sizes, bound on them, precision, iterations, whether the tiles are dealt: few
+# tiles per instance, and bounds above what the instances hold
+LOOSE_DEAL_ROUTES = [(3, "[15] * 20", 60, "F16X2", 3, False), (5, "[15] * 19 + [200]", 200, "F16X2", 3, True),
+                     (2, "[12, 8]", 64, "F16", 2, False), (4, "[40] * 8", 256, "F16", 2, True),
+                     (3, "[22]", 252, "F16X2", 3, False), (3, "[22]", 252, "F16X2", 1, True), (3, "[40]", 252, "F16X2", 3, True)]
+
+
+def test_tiles_are_dealt_by_the_samples_there_are(trace):
+    body = ""
+    for hidden, sizes, bound, prec, gn, _ in LOOSE_DEAL_ROUTES:
+        body += f'h = context(hidden={hidden})\nnote("shape")\nstep(h, {sizes}, c.CROM_PREC_{prec}, gn={gn}, bound={bound})\n'
+    parts = "\n".join(trace(body)).split("shape")[1:]
+    for (hidden, sizes, bound, prec, gn, dealt), part in zip(LOOSE_DEAL_ROUTES, parts, strict=True):
+        ks = kernels(part.splitlines())
+        assert (not any("order" in k for k in ks)) == dealt, (hidden, sizes, bound, prec, gn, ks)
+
+
+# m, r, width, layers, sizes, bound, iterations, the kernel
+FP32_STEP_ROUTES = [(2, 8, 64, 1, "[2181] * 2", 2181, 3, "fwd_fp32"), (2, 2, 64, 1, "[40] * 1400", 40, 2, "fwd_tile"),
+                    (3, 6, 32, 1, "[50] * 388", 71, 3, "fwd_fp32"), (3, 12, 32, 2, "[1768]", 6284, 3, "fwd_fp32"),
+                    (1, 12, 128, 1, "[33] * 34", 62, 1, "fwd_fp32"), (2, 8, 96, 1, "[10286]", 10286, 1, "fwd_fp32"),
+                    (1, 12, 32, 2, "[20000] * 2", 20678, 2, "fwd_fp32"), (1, 12, 32, 2, "[600] * 80", 600, 2, "fwd_tile"), (3, 6, 32, 4, "[150] * 95", 194, 2, "fwd_fp32"),
+                    (3, 6, 64, 4, "[150] * 95", 194, 2, "fwd_tile"), (2, 8, 128, 5, "[300] * 64", 300, 2, "fwd_tile")]
+
+
+def test_fp32_steps_take_the_faster_kernel(trace):
+    body = ""
+    for m, r, width, hidden, sizes, bound, gn, _ in FP32_STEP_ROUTES:
+        body += f'h = context({m}, {r}, {width}, {hidden})\nnote("shape")\nstep(h, {sizes}, c.CROM_PREC_FP32, gn={gn}, r={r}, m={m}, bound={bound})\n'
+    parts = "\n".join(trace(body)).split("shape")[1:]
+    for shape, part in zip(FP32_STEP_ROUTES, parts, strict=True):
+        assert all(shape[-1] in k for k in kernels(part.splitlines())), (shape, kernels(part.splitlines()))
