@@ -235,6 +235,18 @@ cudaError_t launch_step_fp32_noalloc(const crom_ctx* ctx, const crom_step_desc* 
 cudaError_t clear_device(void* p, size_t bytes);
 cudaError_t upload_device(void* p, const void* host, size_t bytes);
 
+// Lets a kernel (of up to 64 bytes of static shared memory) be launched with `smem` bytes of
+// dynamic shared memory.  The limit is the process's, not the launch's: it is set to the
+// largest whenever a launch needs more than the default, never to the launch's own need,
+// which would take it from other threads' launches and from later ones that rely on the
+// default.
+constexpr size_t kMaxDynSmem = 227 * 1024 - 64;
+template <typename Kernel>
+cudaError_t allow_smem(Kernel kernel, size_t smem) {
+  if (smem <= 48 * 1024 - 64) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem);
+}
+
 // Grows a scratch array of the context to n elements, all zero if `zero`.
 template <typename T>
 cudaError_t grow(crom_ctx* ctx, T** buf, size_t* cap, size_t n, bool zero = false) {

@@ -519,7 +519,7 @@ bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 template <typename Kernel>
 cudaError_t launch_cluster(Kernel kernel, const FomParams& p, int nc, int n_batch, int threads, size_t smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(kernel, smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(nc, n_batch);
@@ -585,7 +585,7 @@ cudaError_t launch_2d(const FomParams& p, int n_batch, cudaStream_t s, bool* don
   if (n <= (adv ? kFieldMaxAdv : kFieldMaxHeat) && (!adv || p.steps > 2) && field_pays(kScheme, n, n_batch, p.steps, sms)) {
     const size_t smem = (size_t)(adv ? 4 : 2) * n * n * sizeof(float);
     const auto kernel = kScheme == kHeat && n_batch <= sms ? fom_field_few_kernel : fom_field_kernel<kScheme>;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem(kernel, smem);
     if (e != cudaSuccess) return e;
     *done = true;
     kernel<<<n_batch, std::min(1024, (n * n + 31) / 32 * 32), smem, s>>>(p);
@@ -614,10 +614,8 @@ cudaError_t launch_fom_fused(int kind, int n_batch, int nx, const float* coef, c
     const float r_over = (float)(dt / (dx * dx));
     const size_t smem = (size_t)2 * nx * sizeof(float);
     auto kernel = kind == CROM_FOM_HEAT1D_DIRICHLET ? fom_line_kernel<false> : fom_line_kernel<true>;
-    if (smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(kernel, smem);
+    if (e != cudaSuccess) return e;
     *done = true;
     kernel<<<n_batch, std::min(1024, (nx + 31) / 32 * 32), smem, s>>>(u, coef, nx, n_steps, r_over);
     return cudaGetLastError();

@@ -608,15 +608,13 @@ size_t fwd_smem_bytes(int W, int S, int C, int m, int r, int* LD_out) {
 
 // Which of the forward kernels runs a launch.
 enum FwdKernel { kFwdGeneral = 0, kFwdTile2, kFwdTile3, kFwdSmall };
-constexpr size_t kMaxSmem = 227 * 1024;
+constexpr size_t kMaxSmem = kMaxDynSmem;
 
 cudaError_t launch_fwd(FwdParams& p, FwdKernel kind, dim3 grid, cudaStream_t s) {
   const int W = p.width;
   auto go = [&](auto kernel, int threads, size_t smem) -> cudaError_t {
-    if (smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(kernel, smem);
+    if (e != cudaSuccess) return e;
     kernel<<<grid, threads, smem, s>>>(p);
     return cudaGetLastError();
   };
@@ -643,7 +641,7 @@ cudaError_t launch_fwd(FwdParams& p, FwdKernel kind, dim3 grid, cudaStream_t s) 
     // a chain of launches that each wait for one CTA's solve: the next one's CTAs start and
     // load the decoder meanwhile (200 samples, width 128: 71.5 us a step of two without, 66.8 with;
     // width 64: 53.5 and 52.1)
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kernel, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;

@@ -23,6 +23,7 @@ std::map<const char*, Alloc> g_allocs;
 size_t g_next = 0, g_limit = ~size_t(0), g_streams = 0;
 int g_capturing = 0;  // what cudaStreamIsCapturing answers for streams the library did not make
 std::map<const void*, std::string> g_kernels;
+std::map<const void*, size_t> g_smem;  // dynamic shared memory allowed, where it was set
 std::vector<cudaStream_t> g_own;
 struct Pending {
   cudaStream_t s;
@@ -59,7 +60,11 @@ void done(cudaStream_t s) {
   g_pending.erase(std::remove_if(g_pending.begin(), g_pending.end(), [&](const Pending& p) { return p.s == plain(s); }),
                   g_pending.end());
 }
-cudaError_t launch(const void* f, cudaStream_t s) {
+cudaError_t launch(const void* f, size_t smem, cudaStream_t s) {
+  if (smem > (g_smem.count(f) ? g_smem[f] : 48 * 1024)) {
+    line("TOO MUCH shared memory for " + g_kernels[f]);
+    return cudaErrorInvalidValue;
+  }
   const std::string k = g_kernels.count(f) ? g_kernels[f] : "?";
   line("launch " + k + " stream " + name(s));
   for (const Pending& p : g_pending)
@@ -85,7 +90,13 @@ cudaError_t cudaGetDeviceProperties(cudaDeviceProp* p, int) {
   return cudaSuccess;
 }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 152; return cudaSuccess; }
-cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
+  if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) {
+    if (g_smem.count(f) && (size_t)v < g_smem[f]) line("LOWERED limit of " + g_kernels[f]);
+    g_smem[f] = v;
+  }
+  return cudaSuccess;
+}
 cudaError_t cudaGetLastError(void) { return cudaSuccess; }
 cudaError_t cudaMalloc(void** p, size_t bytes) {
   *p = nullptr;
@@ -154,8 +165,8 @@ cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) {
   *k = reinterpret_cast<cudaKernel_t>(const_cast<void*>(f));
   return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void**, size_t, cudaStream_t s) { return launch(k, s); }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) { return launch(f, c->stream); }
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void**, size_t smem, cudaStream_t s) { return launch(k, smem, s); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) { return launch(f, c->dynamicSmemBytes, c->stream); }
 void __cudaRegisterFunction(void** h, const char* host, char* dev, const char* dname, int lim, uint3* a, uint3* b, dim3* c,
                             dim3* d, int* w) {
   g_kernels[host] = dname;

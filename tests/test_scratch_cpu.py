@@ -326,3 +326,25 @@ def test_fp32_steps_take_the_faster_kernel(trace):
     parts = "\n".join(trace(body)).split("shape")[1:]
     for shape, part in zip(FP32_STEP_ROUTES, parts, strict=True):
         assert all(shape[-1] in k for k in kernels(part.splitlines())), (shape, kernels(part.splitlines()))
+
+
+def test_shared_memory_limits_are_never_lowered(trace):
+    """A kernel's limit is the process's: a call that sets it to its own need takes it from
+    other threads and from later calls within the default (a step of few samples followed
+    by a tangent velocity that needs more than the step did, and less than the default)."""
+    lines = trace("""
+        p = 0x7f0000000000          # not read: no kernel runs
+        h = context(1, 29, 32, 1)
+        step(h, [40] * 4, c.CROM_PREC_FP32, r=29, m=1)
+        ok(c.raw_call("crom_tangent_velocity", h, 1, p, p, 1e-3, p, p, 6, p, S))
+        for r, n in ((8, 200), (2, 40), (16, 100)):
+            step(context(2, r), [n], c.CROM_PREC_FP32, r=r)
+            step(context(2, r), [n] * 60, c.CROM_PREC_FP32, r=r)
+        for kind, n, nb in (("HEAT2D_NEUMANN", 127, 3), ("HEAT2D_NEUMANN", 57, 3), ("HEAT2D_NEUMANN", 100, 1),
+                            ("HEAT2D_NEUMANN", 200, 1), ("HEAT2D_NEUMANN", 64, 1), ("ADVDIFF2D_PERIODIC", 97, 3),
+                            ("ADVDIFF2D_PERIODIC", 57, 3), ("ADVDIFF2D_PERIODIC", 256, 64), ("ADVDIFF2D_PERIODIC", 100, 2)):
+            ok(c.raw_call("crom_fom_step", getattr(c, "CROM_FOM_" + kind), nb, n, n, p, p, p, 1e-9, 20, p, p + (1 << 34), S))
+        for n in (8192, 300, 7000):
+            ok(c.raw_call("crom_fom_step", c.CROM_FOM_HEAT1D_DIRICHLET, 2, n, 1, p, p, p, 1e-9, 20, p, p + (1 << 34), S))
+    """)
+    assert [x for x in lines if x.startswith(("TOO MUCH", "LOWERED"))] == []
