@@ -729,7 +729,12 @@ int pick_samples(int W, int C, int m, int r, int want);
 //    no more rounds of the GPU than (C + 1) / 2 (step: C / 2): its time grows with the rounds, the
 //    general kernel's with the channels (1000 values of width 64: 1.7 times, 45 x 5
 //    channels of 600: 0.9 times).  Width 32 and two layers leave too little to gain in a
-//    second round, three layers in a third.
+//    second round, three layers in a third.  Steps of one layer with up to six codes, and
+//    of two up to width 96 with up to three, take it for instances of at most 16 samples:
+//    longer ones spend more on its rows' tickets and sums than the products gain (one
+//    instance of 213, r = 1, width 128, one layer: 33 against 23 us; 320 steps of one and
+//    two layers: none above 1.02 of the general kernel's time, 0.87 and, as rollouts, 0.91
+//    on average).
 //  * Else the general kernel.
 // (columns: N C; held: a step's, of the samples that there are)
 bool tile_pays(const crom_ctx* ctx, long long columns, int C, bool step, long long held = 0, int n_inst = 0) {
@@ -900,7 +905,9 @@ FwdKernel plan_step(const crom_ctx* ctx, int n_inst, int n_samples, int max_samp
     const FwdKernel k = tile_plan(ctx, n_inst, max_samples, C0, S);
     if (k != kFwdGeneral) return k;
   }
-  for (*S = N > ctx->num_sms ? 2 : 1; *S >= 1; --*S)
+  const int hidden = ctx->desc.hidden;
+  const bool shallow = (hidden == 1 && r <= 6) || (hidden == 2 && r <= 3 && W <= 96);
+  for (*S = N > ctx->num_sms ? 2 : 1; *S >= 1 && (!shallow || max_samples <= 16); --*S)
     if (*S % *PS == 0 && small_fits(W, *S, C0, m, r, ctx->desc.hidden) && small_pays(ctx, N, *S, C0, true)) return kFwdSmall;
   *S = *PS;
   return kFwdGeneral;

@@ -312,7 +312,9 @@ def test_tiles_are_dealt_by_the_samples_there_are(trace):
 
 
 # m, r, width, layers, sizes, bound, iterations, the kernel
-FP32_STEP_ROUTES = [(2, 8, 64, 1, "[2181] * 2", 2181, 3, "fwd_fp32"), (2, 2, 64, 1, "[40] * 1400", 40, 2, "fwd_tile"),
+FP32_STEP_ROUTES = [(1, 1, 128, 1, "[213]", 213, 1, "fwd_fp32"), (1, 1, 128, 1, "[16]", 16, 1, "fwd_small"),
+                    (2, 2, 32, 2, "[47] * 3", 47, 1, "fwd_fp32"), (2, 8, 32, 2, "[47] * 3", 47, 1, "fwd_small"),
+                    (2, 8, 64, 1, "[2181] * 2", 2181, 3, "fwd_fp32"), (2, 2, 64, 1, "[40] * 1400", 40, 2, "fwd_tile"),
                     (3, 6, 32, 1, "[50] * 388", 71, 3, "fwd_fp32"), (3, 12, 32, 2, "[1768]", 6284, 3, "fwd_fp32"),
                     (1, 12, 128, 1, "[33] * 34", 62, 1, "fwd_fp32"), (2, 8, 96, 1, "[10286]", 10286, 1, "fwd_fp32"),
                     (1, 12, 32, 2, "[20000] * 2", 20678, 2, "fwd_fp32"), (1, 12, 32, 2, "[600] * 80", 600, 2, "fwd_tile"), (3, 6, 32, 4, "[150] * 95", 194, 2, "fwd_fp32"),
