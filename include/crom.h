@@ -398,7 +398,8 @@ int crom_train_step(crom_trainer* tr, const float* snaps, const int* pt_idx, con
  * weights; see crom_precision).  Selecting BF16_MIXED the first time allocates its
  * buffers: about (hidden + 2) * B * S * width * 2 bytes, and (hidden - 1) *
  * min(64, ceil(B * S / 64)) * width^2 * 4 for the partial sums of the weight gradients (67 MB
- * at width 256, five layers and 4096 points or more).  Not during stream capture.  Returns CROM_ERR_UNSUPPORTED for other values or shapes. */
+ * at width 256, five layers and 4096 points or more).  Not during stream capture.
+ * Returns CROM_ERR_UNSUPPORTED for other values or shapes. */
 int crom_trainer_set_precision(crom_trainer* tr, int precision);
 /* Encoder only: q [n][r] FP32 for n <= B snapshots [n][P] (initial latent codes). */
 int crom_encode(crom_trainer* tr, int n, const float* snaps, float* q, crom_stream stream);
